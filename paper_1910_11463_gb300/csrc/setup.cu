@@ -195,53 +195,250 @@ __global__ void k_pmap(int n, const int *rowptr, const int *col, const double *v
 }
 
 // ---- lAIR ------------------------------------------------------------------
-__global__ void k_lair_ncand(int nc, const int *cpts, const int *rowptr, const int *col, const uint8_t *S,
-                             const int8_t *cf, int distance, int *ncand) {
-    int ic = blockIdx.x * blockDim.x + threadIdx.x;
-    if (ic >= nc) return;
-    int i = cpts[ic];
+// The pattern of C row i is the set of its strong F neighbours j and, at distance 2,
+// of their strong F neighbours, ascending.  Bit 2 of S marks an entry that is eps_R-
+// strong with an F column, so the passes below test one byte instead of gathering the
+// CF flag of every column (twice), and nf[row] counts a row's marked entries, so the
+// candidates of a C row are counted without visiting its neighbours' rows.  Eight lanes
+// per row: rows hold 7-16 entries on the fine levels, read as one line.
+constexpr uint8_t S_RF = 4;
+
+__global__ void k_mark_rf(int n, const int *rowptr, const int *col, const int8_t *cf, uint8_t *S, int *nf) {
+    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = (int)(tid >> 3), g = (int)(tid & 7);
     int c = 0;
-    for (int p = rowptr[i]; p < rowptr[i + 1]; ++p) {
-        int j = col[p];
-        if ((S[p] & 2) && cf[j] == CF_F) {
-            ++c;
-            if (distance >= 2)
-                for (int q = rowptr[j]; q < rowptr[j + 1]; ++q)
-                    if ((S[q] & 2) && cf[col[q]] == CF_F) ++c;
+    if (i < n)
+        for (int p = rowptr[i] + g; p < rowptr[i + 1]; p += 8) {
+            const uint8_t f = S[p];
+            if ((f & 2) && cf[col[p]] == CF_F) { S[p] = f | S_RF; ++c; }
         }
-    }
-    ncand[ic] = c;
+    for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if (i < n && g == 0) nf[i] = c;
 }
 
-__global__ void k_lair_pattern(int nc, const int *cpts, const int *rowptr, const int *col, const uint8_t *S,
-                               const int8_t *cf, int distance, const int *candptr, int *cand, int *npat) {
-    int ic = blockIdx.x * blockDim.x + threadIdx.x;
-    if (ic >= nc) return;
-    int i = cpts[ic];
-    int *c = cand + candptr[ic];
-    int m = 0;
-    for (int p = rowptr[i]; p < rowptr[i + 1]; ++p) {
-        int j = col[p];
-        if ((S[p] & 2) && cf[j] == CF_F) c[m++] = j;
+// Candidates (with repeats) of every C row.  Rows with more than PAT_BIG of them go to
+// the list of the bitmap kernel (any order: a row's pattern has its own place).
+constexpr int PAT_SMALL = 64, PAT_MID = 256, PAT_BIG = 1024;
+
+__global__ void k_lair_ncand(int nc, const int *cpts, const int *rowptr, const int *col, const uint8_t *S,
+                             const int *nf, int distance, int *ncand, int *big, int *nbig) {
+    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int ic = (int)(tid >> 3), g = (int)(tid & 7);
+    int c = 0;
+    if (ic < nc) {
+        const int i = cpts[ic];
+        if (distance < 2) c = g == 0 ? nf[i] : 0;
+        else
+            for (int p = rowptr[i] + g; p < rowptr[i + 1]; p += 8)
+                if (S[p] & S_RF) c += 1 + nf[col[p]];
     }
-    if (distance >= 2) {
-        int m1 = m;
-        for (int t = 0; t < m1; ++t) {
-            int j = c[t];
-            for (int q = rowptr[j]; q < rowptr[j + 1]; ++q)
-                if ((S[q] & 2) && cf[col[q]] == CF_F) c[m++] = col[q];
+    for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if (ic < nc && g == 0) {
+        ncand[ic] = c;
+        if (distance >= 2 && c > PAT_BIG) big[atomicAdd(nbig, 1)] = ic;
+    }
+}
+
+// distance 1: the marked entries of the C row, in order (ncand is then the pattern's
+// size); eight lanes per row
+__global__ void k_lair_pattern1(int nc, const int *cpts, const int *rowptr, const int *col, const uint8_t *S,
+                                const int *candptr, int *cand) {
+    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int ic = (int)(tid >> 3), g = (int)(tid & 7);
+    const int lane = threadIdx.x & 31, sh = lane & ~7;
+    int p0 = 0, p1 = 0, out = 0;
+    if (ic < nc) {
+        const int i = cpts[ic];
+        p0 = rowptr[i];
+        p1 = rowptr[i + 1];
+        out = candptr[ic];
+    }
+    int len = p1 - p0;
+    for (int o = 16; o > 0; o >>= 1) len = max(len, __shfl_xor_sync(0xffffffffu, len, o));
+    for (int t = 0; t < len; t += 8) {
+        const int p = p0 + t + g;
+        const bool in = p < p1 && (S[p] & S_RF);
+        const unsigned m = (__ballot_sync(0xffffffffu, in) >> sh) & 0xffu;
+        if (in) cand[out + __popc(m & ((1u << g) - 1u))] = col[p];
+        out += __popc(m);
+    }
+}
+
+// distance 2: G lanes per C row with lo < ncand <= hi.  The candidates go into a hash
+// table of CAP >= 2 hi slots in shared memory (so it is at most half full), the distinct
+// ones are compacted and written at their rank.  A thread per row with an insertion sort
+// of its candidates in global memory took O(ncand^2) dependent accesses: 5.3 ms a level on
+// an 18^3 x 6 tet matrix (rows of 120 entries, thousands of candidates), where the three
+// classes and the bitmap kernel below now take 0.1 ms.  With few candidates (G = 8) a lane
+// walks a neighbour's short row; a warp (G = 32) takes the neighbours' rows one after the
+// other, lanes across the row.  A warp looks at rb rows' counts together and then takes
+// the rows of its class, since most rows of a fine level belong to the smallest class.
+template <int G, int CAP, int HI>
+__global__ void __launch_bounds__(128) k_lair_pattern2(int nc, const int *cpts, const int *rowptr, const int *col,
+                                                       const uint8_t *S, const int *candptr, const int *ncand, int lo,
+                                                       int rb, int *cand, int *npat) {
+    extern __shared__ int psm[];
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, g = lane % G, q = lane / G;
+    const int grp = threadIdx.x / G;   // group of the block
+    const unsigned gmask = G == 32 ? FULL : (((1u << (G & 31)) - 1u) << (q * G));
+    int *keys = psm + grp * (CAP + HI), *list = keys + CAP;
+    auto insert = [&](int c) {
+        unsigned h = ((unsigned)c * 2654435761u) & (CAP - 1);
+        while (true) {   // ends: at most HI <= CAP / 2 distinct columns
+            const int prev = atomicCAS(&keys[h], -1, c);
+            if (prev == -1 || prev == c) return;
+            h = (h + 1) & (CAP - 1);
         }
-        for (int a = 1; a < m; ++a) {   // insertion sort, then unique
-            int v = c[a], b = a;
-            while (b > 0 && c[b - 1] > v) { c[b] = c[b - 1]; --b; }
-            c[b] = v;
+    };
+    // the pattern of row ic (mine: it belongs to the class; whole warps arrive here)
+    auto row = [&](int ic, bool mine) {
+        for (int t = g; t < CAP; t += G) keys[t] = -1;
+        __syncwarp();
+        int p0 = 0, p1 = 0;
+        if (mine) {
+            const int i = cpts[ic];
+            p0 = rowptr[i];
+            p1 = rowptr[i + 1];
         }
+        if (G < 32) {
+            for (int p = p0 + g; p < p1; p += G) {
+                if (!(S[p] & S_RF)) continue;
+                const int j = col[p];
+                insert(j);
+                const int e = rowptr[j + 1];
+                for (int r = rowptr[j]; r < e; r += 4) {   // four entries' loads before their insertions
+                    int c[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) c[u] = (r + u < e && (S[r + u] & S_RF)) ? col[r + u] : -1;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (c[u] >= 0) insert(c[u]);
+                }
+            }
+        } else {
+            for (int t = p0; t < p1; t += 32) {
+                const int p = t + lane;
+                const bool in = p < p1 && (S[p] & S_RF);
+                int j = 0, rs = 0, re = 0;
+                if (in) {
+                    j = col[p];
+                    rs = rowptr[j];
+                    re = rowptr[j + 1];
+                    insert(j);
+                }
+                for (unsigned b = __ballot_sync(FULL, in); b; b &= b - 1) {
+                    const int src = __ffs(b) - 1;
+                    const int s0 = __shfl_sync(FULL, rs, src), s1 = __shfl_sync(FULL, re, src);
+                    for (int r = s0 + lane; r < s1; r += 32)
+                        if (S[r] & S_RF) insert(col[r]);
+                }
+            }
+        }
+        __syncwarp();
         int u = 0;
-        for (int a = 0; a < m; ++a)
-            if (u == 0 || c[u - 1] != c[a]) c[u++] = c[a];
-        m = u;
+        for (int t0 = 0; t0 < CAP; t0 += G) {
+            const int k = keys[t0 + g];
+            const unsigned b = __ballot_sync(FULL, k >= 0) & gmask;
+            if (k >= 0) list[u + __popc(b & ((1u << lane) - 1u))] = k;
+            u += __popc(b);
+        }
+        __syncwarp();
+        if (mine) {
+            const int base = candptr[ic];
+            for (int e = g; e < u; e += G) {
+                const int k = list[e];
+                int rank = 0;
+                for (int f = 0; f < u; ++f) rank += list[f] < k;
+                cand[base + rank] = k;
+            }
+            if (g == 0) npat[ic] = u;
+        }
+        __syncwarp();
+    };
+    if (G < 32) {
+        const int ic = blockIdx.x * (128 / G) + grp;
+        const int m = ic < nc ? ncand[ic] : HI + 1;
+        const bool mine = m <= HI && m >= lo;
+        if (__any_sync(FULL, mine)) row(ic, mine);
+    } else {
+        const long long r0 = (blockIdx.x * 4LL + grp) * rb;
+        const int m = (lane < rb && r0 + lane < nc) ? ncand[r0 + lane] : HI + 1;
+        for (unsigned b = __ballot_sync(FULL, m <= HI && m >= lo); b; b &= b - 1) row((int)r0 + __ffs(b) - 1, true);
     }
-    npat[ic] = m;
+}
+
+// distance 2, rows with more than PAT_BIG candidates: a CTA per row marks the candidates
+// in a bitmap of PAT_WIN columns (32 KB of shared memory), whose set bits come out
+// ascending and distinct; neighbourhoods spread over more columns take further windows
+// over the row's column range.  Grid-stride over the list k_lair_ncand filled.
+constexpr int PAT_WIN = 1 << 18;
+
+__global__ void __launch_bounds__(256) k_lair_pattern2_big(const int *big, const int *nbig, const int *cpts,
+                                                           const int *rowptr, const int *col, const uint8_t *S,
+                                                           const int *candptr, int *cand, int *npat) {
+    __shared__ unsigned bits[PAT_WIN / 32];
+    __shared__ int red[2][8], wsum[8];
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int n = *nbig;
+    for (int k = blockIdx.x; k < n; k += gridDim.x) {
+        const int ic = big[k], i = cpts[ic], p0 = rowptr[i], p1 = rowptr[i + 1];
+        // every candidate to f: a warp per marked neighbour, lanes across its row
+        auto visit = [&](auto f) {
+            for (int p = p0 + w; p < p1; p += 8) {
+                if (!(S[p] & S_RF)) continue;
+                const int j = col[p];
+                if (lane == 0) f(j);
+                for (int r = rowptr[j] + lane; r < rowptr[j + 1]; r += 32)
+                    if (S[r] & S_RF) f(col[r]);
+            }
+        };
+        int lo = 0x7fffffff, hi = -1;
+        visit([&](int c) { lo = min(lo, c); hi = max(hi, c); });
+        for (int o = 16; o > 0; o >>= 1) {
+            lo = min(lo, __shfl_xor_sync(FULL, lo, o));
+            hi = max(hi, __shfl_xor_sync(FULL, hi, o));
+        }
+        if (lane == 0) { red[0][w] = lo; red[1][w] = hi; }
+        __syncthreads();
+        for (int t = 0; t < 8; ++t) { lo = min(lo, red[0][t]); hi = max(hi, red[1][t]); }
+        int out = candptr[ic];
+        const int out0 = out;
+        for (long long c0 = lo; c0 <= hi; c0 += PAT_WIN) {
+            const int nw = (int)((min((long long)hi - c0 + 1, (long long)PAT_WIN) + 31) / 32);   // words in use
+            const int per = (nw + 255) / 256;                                                    // words per thread
+            for (int t = threadIdx.x; t < nw; t += 256) bits[t] = 0u;
+            __syncthreads();
+            visit([&](int c) {
+                const long long d = c - c0;
+                if (d >= 0 && d < PAT_WIN) atomicOr(&bits[d >> 5], 1u << (d & 31));
+            });
+            __syncthreads();
+            const int t0 = min((int)threadIdx.x * per, nw), t1 = min(t0 + per, nw);
+            int cnt = 0;
+            for (int t = t0; t < t1; ++t) cnt += __popc(bits[t]);
+            int inc = cnt;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(FULL, inc, o);
+                if (lane >= o) inc += v;
+            }
+            if (lane == 31) wsum[w] = inc;
+            __syncthreads();
+            int before = inc - cnt, tot = 0;
+            for (int t = 0; t < 8; ++t) {
+                if (t < w) before += wsum[t];
+                tot += wsum[t];
+            }
+            int at = out + before;
+            for (int t = t0; t < t1; ++t)
+                for (unsigned b = bits[t]; b; b &= b - 1) cand[at++] = (int)(c0 + 32LL * t) + __ffs(b) - 1;
+            out += tot;
+            __syncthreads();   // bits, wsum and red are written again
+        }
+        if (threadIdx.x == 0) npat[ic] = out - out0;
+        __syncthreads();
+    }
 }
 
 // lAIR systems binned by size: a thread per system up to 8 unknowns (bins of 4, 6
@@ -1495,17 +1692,47 @@ void build_hierarchy(Hier &h) {
         // ---- lAIR -----------------------------------------------------------
         const int rdist = prm.nair ? 2 : prm.distance;   // nAIR degree 1 uses the distance-2 pattern
         int *ncand = dmalloc<int>(nc, s);
-        k_lair_ncand<<<blocks_for(nc, BS), BS, 0, s>>>(nc, L.cpts, L.rowptr, L.col, S, L.cf, rdist, ncand);
+        int *nf = dmalloc<int>(n, s);
+        k_mark_rf<<<blocks_for(8LL * n, BS), BS, 0, s>>>(n, L.rowptr, L.col, L.cf, S, nf);
         PR_LAUNCH();
+        int *pbig = dmalloc<int>(rdist >= 2 ? nc + 1 : 1, s);   // [count, rows with many candidates]
+        PR_CUDA(cudaMemsetAsync(pbig, 0, sizeof(int), s));
+        k_lair_ncand<<<blocks_for(8LL * nc, BS), BS, 0, s>>>(nc, L.cpts, L.rowptr, L.col, S, nf, rdist, ncand,
+                                                             pbig + 1, pbig);
+        PR_LAUNCH();
+        dfree(nf, s);
         int *candptr = dmalloc<int>(nc + 1, s);
         long long ncandt = scan_exclusive(ncand, candptr, nc, s);
         int *cand = dmalloc<int>(ncandt, s);
-        int *npat = ncand;   // reuse
-        k_lair_pattern<<<blocks_for(nc, BS), BS, 0, s>>>(nc, L.cpts, L.rowptr, L.col, S, L.cf, rdist, candptr, cand,
-                                                         npat);
-        PR_LAUNCH();
+        int *npat = ncand;   // distance 1: the candidates are the pattern
         int *zr = dmalloc<int>(nc + 1, s);
-        long long nz = scan_exclusive(npat, zr, nc, s);
+        long long nz = ncandt;
+        if (rdist < 2) {
+            k_lair_pattern1<<<blocks_for(8LL * nc, BS), BS, 0, s>>>(nc, L.cpts, L.rowptr, L.col, S, candptr, cand);
+            PR_LAUNCH();
+            PR_CUDA(cudaMemcpyAsync(zr, candptr, sizeof(int) * (nc + 1), cudaMemcpyDeviceToDevice, s));
+        } else {
+            // one launch per size class over all rows (a row of another class costs its
+            // count), no partition and no host read
+            npat = dmalloc<int>(nc, s);
+            const int rb = std::max(1, std::min(32, nc / (152 * 48)));   // rows per warp, enough warps to fill the chip
+            auto pat2 = [&](auto kern, int G, int cap, int lo, int hi) {
+                const size_t sm = (size_t)(128 / G) * (cap + hi) * sizeof(int);
+                const int rows = G < 32 ? 128 / G : 4 * rb;
+                kern<<<blocks_for(nc, rows), 128, sm, s>>>(nc, L.cpts, L.rowptr, L.col, S, candptr, ncand, lo, rb, cand,
+                                                          npat);
+                PR_LAUNCH();
+            };
+            pat2(k_lair_pattern2<8, 2 * PAT_SMALL, PAT_SMALL>, 8, 2 * PAT_SMALL, 0, PAT_SMALL);
+            pat2(k_lair_pattern2<32, 2 * PAT_MID, PAT_MID>, 32, 2 * PAT_MID, PAT_SMALL + 1, PAT_MID);
+            pat2(k_lair_pattern2<32, 2 * PAT_BIG, PAT_BIG>, 32, 2 * PAT_BIG, PAT_MID + 1, PAT_BIG);
+            k_lair_pattern2_big<<<std::min<unsigned>(nc, 152u * 6u), 256, 0, s>>>(pbig + 1, pbig, L.cpts, L.rowptr,
+                                                                                 L.col, S, candptr, cand, npat);
+            PR_LAUNCH();
+            dfree(ncand, s);
+            nz = scan_exclusive(npat, zr, nc, s);
+        }
+        dfree(pbig, s);
         int *zc = dmalloc<int>(nz, s);
         double *zv = dmalloc<double>(nz, s);
         int *keep = dmalloc<int>(nc, s);
@@ -1597,7 +1824,7 @@ void build_hierarchy(Hier &h) {
             dfree(zr, s);
         }
         L.zrowptr = zr2; L.zcol = zc; L.zval = zv; L.nnzZ = nz2;
-        dfree(keep, s); dfree(cand, s); dfree(candptr, s); dfree(ncand, s);
+        dfree(keep, s); dfree(cand, s); dfree(candptr, s); dfree(npat, s);
         dfree(S, s);
 
         PR_CUDA(cudaEventRecord(ev[2], s));

@@ -1,0 +1,84 @@
+"""Setup kernels at the sizes where their classes meet, bit for bit against the oracle."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pair():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__ as g
+    g.build()
+    from paper_1910_11463_gb300 import pair as P
+    return P
+
+
+def _matrix(n, rows, seed, spread=None):
+    """CSR matrix with unit diagonal; rows: row -> number of off-diagonal entries (others
+    hold none), columns drawn within `spread` of the row (the whole matrix: None), values
+    small enough for a stable local solve."""
+    g = np.random.default_rng(seed)
+    rp, ci, va = [0], [], []
+    for i in range(n):
+        k = rows(i)
+        c = np.zeros(0, np.int64)
+        if k:
+            lo, hi = (0, n) if spread is None else (max(0, i - spread), min(n, i + spread + 1))
+            c = np.unique(g.integers(lo, hi, k))
+            c = c[c != i]
+        c = np.sort(np.append(c, i))
+        v = np.where(c == i, 1.0, g.uniform(-1.0, 1.0, c.size) / max(1, c.size))
+        rp.append(rp[-1] + c.size)
+        ci.append(c)
+        va.append(v)
+    return np.array(rp, np.int32), np.concatenate(ci).astype(np.int32), np.concatenate(va)
+
+
+def _check(pair, rp, ci, va, **kw):
+    G = pair.Hierarchy([tuple(torch.as_tensor(a, device="cuda") for a in (rp, ci, va))],
+                       pair.default_air_params(precision=0, **kw))
+    H = O.Hierarchy(rp, ci, va, O.default_params(**kw))
+    assert G.nlevels(0) == H.nlev
+    for l in range(H.nlev):
+        a, b = G.level(0, l), H.level(l)
+        assert np.array_equal(a.rowptr, b.rowptr) and np.array_equal(a.col, b.col), l
+        assert np.array_equal(a.val.view(np.uint64), b.val.view(np.uint64)), l
+        if not a.coarsest:
+            assert np.array_equal(a.cf, b.cf) and np.array_equal(a.pmap, b.pmap), l
+            assert np.array_equal(a.zrowptr, b.zrowptr) and np.array_equal(a.zcol, b.zcol), l
+            assert np.array_equal(a.zval.view(np.uint64), b.zval.view(np.uint64)), l
+    return H
+
+
+@pytest.mark.parametrize("distance,entries,n", [
+    (1, 3, 100), (1, 9, 333), (1, 40, 500),      # lanes per row: under, over and far over eight entries
+    (2, 3, 64), (2, 8, 400),                     # up to 64 candidates
+    (2, 14, 700),                                # up to 256
+    (2, 30, 900),                                # up to 1024
+    (2, 45, 500),                               # the bitmap
+])
+def test_lair_pattern_classes(pair, distance, entries, n):
+    rp, ci, va = _matrix(n, lambda i: entries if i % 3 else max(1, entries // 4), 5 + entries)
+    _check(pair, rp, ci, va, distance=distance, theta=0.5, max_levels=2, max_coarse=10)
+
+
+def test_lair_pattern_windows(pair):
+    """More than 1024 candidates spread over more columns than one bitmap window holds."""
+    n = 600_000
+    rp, ci, va = _matrix(n, lambda i: 40 if i % 12_000 == 0 else (40 if i % 6_007 == 1 else 0), 3)
+    # dense rows point at one another across the matrix
+    dense = np.array([i for i in range(n) if i % 12_000 == 0 or i % 6_007 == 1])
+    g = np.random.default_rng(9)
+    for i in dense:
+        s, e = rp[i], rp[i + 1]
+        k = e - s - 1
+        c = np.sort(np.append(g.choice(dense[dense != i], size=k, replace=False), i))
+        ci[s:e] = c
+        va[s:e] = np.where(c == i, 1.0, g.uniform(0.5, 1.0, k + 1) / (4 * k))
+    _check(pair, rp, ci, va, distance=2, theta=0.5, eps_R=0.001, max_levels=2)
