@@ -53,8 +53,6 @@ __device__ __forceinline__ V4<double> load4(const double *p) {
     return {a.x, a.y, b.x, b.y};
 }
 
-// Off-diagonal part of row (m, e, a) of the hex block operator applied to v
-// (v points at direction m's vector).  Returns sum_faces sum_t A v.
 // Level-0 block kernels run on a 3-D grid: x = tiles of 32 elements along a
 // mesh row (8 rows each, 256 threads), y = iy + n iz, z = direction, so the
 // element coordinates come from block indices.
@@ -76,26 +74,45 @@ __device__ __forceinline__ HexRow hex_row(int n) {
     return r;
 }
 
-template <class T, class TV>
-__device__ __forceinline__ T bsr_offdiag(int n, long long E, int m, int e, int a, const int *idx, const int8_t *dsign,
-                                         const T *vals, const TV *v) {
+// Upwind face rows of row (m, e, a): values and neighbours (constants of a solve),
+// loaded ahead of the vector they multiply
+template <class T>
+struct HexFaces {
+    V4<T> w[3];
+    int off[3];   // first DOF of the upwind element across axis d, -1: none
+    int o[3];     // its face: node bit along d
+};
+
+template <class T>
+__device__ __forceinline__ HexFaces<T> hex_faces(int n, long long E, int m, int e, int a, const int *idx,
+                                                 const int8_t *dsign, const T *vals, bool need = true) {
     const int stride[3] = {1, n, n * n};
-    T acc = T(0);
     const T *base = vals + (((long long)m * E + e) * 3) * 32 + a * 4;
+    HexFaces<T> f;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        int sg = dsign[3 * m + d];
-        if (sg == 0) continue;
-        bool has = sg > 0 ? idx[d] > 0 : idx[d] < n - 1;
-        if (!has) continue;
-        int ep = sg > 0 ? e - stride[d] : e + stride[d];
-        int o = sg > 0 ? 1 : 0;
-        V4<T> w = load4(base + d * 32);
-        const TV *xb = v + 8LL * ep;
-        acc += w.x * (T)xb[face_node(d, o, 0)];
-        acc += w.y * (T)xb[face_node(d, o, 1)];
-        acc += w.z * (T)xb[face_node(d, o, 2)];
-        acc += w.w * (T)xb[face_node(d, o, 3)];
+        const int sg = dsign[3 * m + d];
+        const bool has = need && (sg > 0 ? idx[d] > 0 : (sg < 0 && idx[d] < n - 1));
+        f.off[d] = has ? 8 * (sg > 0 ? e - stride[d] : e + stride[d]) : -1;
+        f.o[d] = sg > 0 ? 1 : 0;
+        f.w[d] = has ? load4(base + d * 32) : V4<T>{T(0), T(0), T(0), T(0)};
+    }
+    return f;
+}
+
+// off-diagonal part of the row applied to v (direction m's vector)
+template <class T, class TV>
+__device__ __forceinline__ T hex_apply(const HexFaces<T> &f, const TV *v) {
+    T acc = T(0);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        if (f.off[d] < 0) continue;
+        const TV *xb = v + f.off[d];
+        const int o = f.o[d];
+        acc += f.w[d].x * (T)xb[face_node(d, o, 0)];
+        acc += f.w[d].y * (T)xb[face_node(d, o, 1)];
+        acc += f.w[d].z * (T)xb[face_node(d, o, 2)];
+        acc += f.w[d].w * (T)xb[face_node(d, o, 3)];
     }
     return acc;
 }
@@ -133,24 +150,27 @@ __device__ __forceinline__ double block_sum(double v) {
 }
 
 // ---- level-0 FP64 residual --------------------------------------------------
-template <class T>
+template <class T, bool AHEAD>
 __global__ void __launch_bounds__(BS) k_res0_bsr(int n, int N, const int8_t *dsign, const double *bsr64,
                                                  const double *b, const double *x, T *r, float *r2,
                                                  double *partials, int maxblk, const int *active, int zero_x) {
-    pdl_begin();
     HexRow q = hex_row(n);
-    if (active && !active[q.m]) return;
+    pdl_wait_if<!AHEAD>();
+    if (!AHEAD && active && !active[q.m]) return;
+    const HexFaces<double> fc = hex_faces<double>(n, (long long)N / 8, q.m, q.e, q.a, q.idx, dsign, bsr64,
+                                                  q.valid && !zero_x);
+    pdl_wait_if<AHEAD>();
+    if (AHEAD && active && !active[q.m]) return;
     constexpr bool F32 = std::is_same<T, float>::value;
     double s2 = 0.0;
     float s2f = 0.0f;
-    long long E = (long long)N / 8;
     if (q.valid) {
         long long gi = (long long)q.m * N + 8LL * q.e + q.a;
         // x = 0 (a solve's first residual): r = b, no operator read
         double acc = b[gi];
         if (!zero_x) {
             acc -= x[gi];
-            acc -= bsr_offdiag<double, double>(n, E, q.m, q.e, q.a, q.idx, dsign, bsr64, x + (long long)q.m * N);
+            acc -= hex_apply<double, double>(fc, x + (long long)q.m * N);
         }
         T rt = (T)acc;
         r[gi] = rt;
@@ -205,34 +225,39 @@ __device__ __forceinline__ void load_dd4(const float2 *p, float2 *w) {
 
 // Level-0 residual of the block form in double-float: r = b - x - sum_faces A x_nbr,
 // cast to FP32 for the cycle, FP32 squares for the norm (as in k_res0_bsr<float>)
+template <bool AHEAD>
 __global__ void __launch_bounds__(BS) k_res0_bsr_dd(int n, int N, const int8_t *dsign, const float2 *vals,
                                                     const float2 *b, const float2 *x, float *r, float *r2,
                                                     double *partials, int maxblk, const int *active) {
-    pdl_begin();
     HexRow q = hex_row(n);
-    if (active && !active[q.m]) return;
+    pdl_wait_if<!AHEAD>();
+    if (!AHEAD && active && !active[q.m]) return;
+    const int stride[3] = {1, n, n * n};
+    const float2 *base = vals + (((long long)q.m * (N / 8) + q.e) * 3) * 32 + q.a * 4;
+    float2 w[3][4];
+    int off[3], o[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const int sg = dsign[3 * q.m + d];
+        const bool has = q.valid && (sg > 0 ? q.idx[d] > 0 : (sg < 0 && q.idx[d] < n - 1));
+        off[d] = has ? 8 * (sg > 0 ? q.e - stride[d] : q.e + stride[d]) : -1;
+        o[d] = sg > 0 ? 1 : 0;
+        if (has) load_dd4(base + d * 32, w[d]);
+    }
+    pdl_wait_if<AHEAD>();
+    if (AHEAD && active && !active[q.m]) return;
     float s2f = 0.0f;
     if (q.valid) {
-        const long long E = (long long)N / 8;
         const long long gi = (long long)q.m * N + 8LL * q.e + q.a;
         const float2 bi = b[gi], xi = x[gi];
         const float2 *xm = x + (long long)q.m * N;
-        const int stride[3] = {1, n, n * n};
-        const float2 *base = vals + (((long long)q.m * E + q.e) * 3) * 32 + q.a * 4;
         float2 acc = make_float2(0.0f, 0.0f);
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            const int sg = dsign[3 * q.m + d];
-            if (sg == 0) continue;
-            const bool has = sg > 0 ? q.idx[d] > 0 : q.idx[d] < n - 1;
-            if (!has) continue;
-            const int ep = sg > 0 ? q.e - stride[d] : q.e + stride[d];
-            const int o = sg > 0 ? 1 : 0;
-            float2 w[4];
-            load_dd4(base + d * 32, w);
-            const float2 *xb = xm + 8LL * ep;
+            if (off[d] < 0) continue;
+            const float2 *xb = xm + off[d];
 #pragma unroll
-            for (int t = 0; t < 4; ++t) dd_fma_acc(acc, w[t], xb[face_node(d, o, t)]);
+            for (int t = 0; t < 4; ++t) dd_fma_acc(acc, w[d][t], xb[face_node(d, o[d], t)]);
         }
         acc = fast_two_sum(acc.x, acc.y);
         // (b - x) - acc in pairs
@@ -259,22 +284,59 @@ __global__ void k_dd_join(long long n, const float2 *a, double *out) {
     if (i < n) out[i] = (double)a[i].x + (double)a[i].y;
 }
 
+// A CSR row's dot product: CSR_U entries' loads together (the first ones before the
+// kernel's wait), then their gathers, then the adds in entry order
+constexpr int CSR_U = 8;
 template <class T>
+struct CsrRow {
+    int p0, p1, c[CSR_U];
+    T v[CSR_U];
+    __device__ __forceinline__ void load(int p, const int *col, const T *val) {
+#pragma unroll
+        for (int u = 0; u < CSR_U; ++u) {
+            c[u] = p + u < p1 ? col[p + u] : -1;
+            v[u] = p + u < p1 ? val[p + u] : T(0);
+        }
+    }
+    __device__ __forceinline__ T dot(const int *col, const T *val, const T *x) {
+        T acc = T(0);
+        for (int p = p0; p < p1; p += CSR_U) {
+            if (p != p0) load(p, col, val);
+            T g[CSR_U];
+#pragma unroll
+            for (int u = 0; u < CSR_U; ++u) g[u] = c[u] >= 0 ? x[c[u]] : T(0);
+#pragma unroll
+            for (int u = 0; u < CSR_U; ++u)
+                if (c[u] >= 0) acc += v[u] * g[u];
+        }
+        return acc;
+    }
+};
+
+template <class T, bool AHEAD>
 __global__ void __launch_bounds__(BS) k_res0_csr(const int *row0, const int *nrow, const int *rowptr, const int *col,
                                                  const double *val, const double *b, const double *x, T *r,
                                                  float *r2, double *partials, int maxblk, const int *active,
                                                  int zero_x) {
-    pdl_begin();
-    int m = blockIdx.y;
-    if (active && !active[m]) return;
-    int li = blockIdx.x * blockDim.x + threadIdx.x;
+    const int m = blockIdx.y;
+    pdl_wait_if<!AHEAD>();
+    if (!AHEAD && active && !active[m]) return;
+    const int li = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool has = li < nrow[m];
+    const int i = row0[m] + li;
+    CsrRow<double> A;
+    A.p0 = A.p1 = 0;
+    if (has && !zero_x) {   // x = 0 (a solve's first residual): r = b, no operator read
+        A.p0 = rowptr[i];
+        A.p1 = rowptr[i + 1];
+    }
+    A.load(A.p0, col, val);
+    pdl_wait_if<AHEAD>();
+    if (AHEAD && active && !active[m]) return;
     double s2 = 0.0;
-    if (li < nrow[m]) {
-        int i = row0[m] + li;
-        double acc = 0.0;
-        if (!zero_x)   // x = 0 (a solve's first residual): r = b, no operator read
-            for (int p = rowptr[i]; p < rowptr[i + 1]; ++p) acc += val[p] * x[col[p]];
-        acc = b[i] - acc;
+    if (has) {
+        const double bi = b[i];
+        const double acc = bi - A.dot(col, val, x);
         r[i] = (T)acc;
         if (r2) r2[i] = (float)acc;
         s2 = acc * acc;
@@ -288,18 +350,21 @@ __global__ void __launch_bounds__(BS) k_res0_csr(const int *row0, const int *nro
 // by FP32 V-cycles; between cycles the FP32 residual r32 - A d32 is the next
 // cycle's right-hand side.  Block form: identity diagonal, element-ordered FP32
 // face blocks (bsr32), the same grid and norm partials as the outer residual.
+template <bool AHEAD>
 __global__ void __launch_bounds__(BS) k_res32_bsr(int n, int N, const int8_t *dsign, const float *bsr32,
                                                   const float *r0, const float *d, float *r, double *partials,
                                                   int maxblk, const int *active) {
-    pdl_begin();
     HexRow q = hex_row(n);
-    if (active && !active[q.m]) return;
+    pdl_wait_if<!AHEAD>();
+    if (!AHEAD && active && !active[q.m]) return;
+    const HexFaces<float> fc = hex_faces<float>(n, (long long)N / 8, q.m, q.e, q.a, q.idx, dsign, bsr32, q.valid);
+    pdl_wait_if<AHEAD>();
+    if (AHEAD && active && !active[q.m]) return;
     float s2f = 0.0f;
     if (q.valid) {
-        const long long E = (long long)N / 8;
         const long long gi = (long long)q.m * N + 8LL * q.e + q.a;
         const float r0i = r0[gi], di = d[gi];
-        const float acc = bsr_offdiag<float, float>(n, E, q.m, q.e, q.a, q.idx, dsign, bsr32, d + (long long)q.m * N);
+        const float acc = hex_apply<float, float>(fc, d + (long long)q.m * N);
         const float rt = r0i - (di + acc);
         r[gi] = rt;
         s2f = rt * rt;
@@ -309,19 +374,29 @@ __global__ void __launch_bounds__(BS) k_res32_bsr(int n, int N, const int8_t *ds
 }
 
 // CSR level 0 (diagonal stored): r = r0 - A d with FP32 values
+template <bool AHEAD>
 __global__ void __launch_bounds__(BS) k_res32_csr(const int *row0, const int *nrow, const int *rowptr, const int *col,
                                                   const float *val, const float *r0, const float *d, float *r,
                                                   double *partials, int maxblk, const int *active) {
-    pdl_begin();
     const int m = blockIdx.y;
-    if (active && !active[m]) return;
+    pdl_wait_if<!AHEAD>();
+    if (!AHEAD && active && !active[m]) return;
     const int li = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool has = li < nrow[m];
+    const int i = row0[m] + li;
+    CsrRow<float> A;
+    A.p0 = A.p1 = 0;
+    if (has) {
+        A.p0 = rowptr[i];
+        A.p1 = rowptr[i + 1];
+    }
+    A.load(A.p0, col, val);
+    pdl_wait_if<AHEAD>();
+    if (AHEAD && active && !active[m]) return;
     float s2f = 0.0f;
-    if (li < nrow[m]) {
-        const int i = row0[m] + li;
-        float acc = 0.0f;
-        for (int p = rowptr[i]; p < rowptr[i + 1]; ++p) acc += val[p] * d[col[p]];
-        const float rt = r0[i] - acc;
+    if (has) {
+        const float r0i = r0[i];
+        const float rt = r0i - A.dot(col, val, d);
         r[i] = rt;
         s2f = rt * rt;
     }
@@ -481,50 +556,20 @@ __global__ void k_sumsq_rows(const int *row0, const int *nrow, const double *v, 
 // added in ascending entry order.
 constexpr int SELL_U = 8;
 
-template <class T, int G, int U>
-__device__ __forceinline__ T sell_dot(int base, int len, int g, const int *col, const T *val, const T *in) {
-    T acc = T(0);
-    for (int j0 = g; j0 < len; j0 += U * G) {
-        int c[U];
-        T v[U], x[U];
+// One pass of U entries per lane from j0: columns (C16: 16-bit offsets from row r) and
+// values, predicated on the row's length
+template <class T, int G, int U, bool C16>
+__device__ __forceinline__ void sell_load(int base, int len, int j0, int r, const int *col, const short *col16,
+                                          const T *val, int (&c)[U], T (&v)[U]) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const bool ok = j0 + u * G < len;
-            c[u] = ok ? __ldcs(col + base + 32 * (j0 + u * G)) : 0;
-            v[u] = ok ? __ldcs(val + base + 32 * (j0 + u * G)) : T(0);
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) x[u] = j0 + u * G < len ? in[c[u]] : T(0);
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (j0 + u * G < len) acc += v[u] * x[u];
+    for (int u = 0; u < U; ++u) {
+        const bool ok = j0 + u * G < len;
+        const int at = base + 32 * (j0 + u * G);
+        if (C16) c[u] = ok ? r + (int)__ldcs(col16 + at) : 0;
+        else c[u] = ok ? __ldcs(col + at) : 0;
+        v[u] = ok ? __ldcs(val + at) : T(0);
     }
-    return acc;
 }
-
-// the same with 16-bit column offsets from the row r (col = r + offset)
-template <class T, int G, int U>
-__device__ __forceinline__ T sell_dot16(int base, int len, int g, int r, const short *col16, const T *val,
-                                        const T *in) {
-    T acc = T(0);
-    for (int j0 = g; j0 < len; j0 += U * G) {
-        int c[U];
-        T v[U], x[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const bool ok = j0 + u * G < len;
-            c[u] = ok ? r + (int)__ldcs(col16 + base + 32 * (j0 + u * G)) : 0;
-            v[u] = ok ? __ldcs(val + base + 32 * (j0 + u * G)) : T(0);
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) x[u] = j0 + u * G < len ? in[c[u]] : T(0);
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (j0 + u * G < len) acc += v[u] * x[u];
-    }
-    return acc;
-}
-
 
 enum SellMode : int { SM_F = 0, SM_C = 1, SM_C_FINAL = 2, SM_RESTRICT = 3 };
 
@@ -561,33 +606,64 @@ struct SellJob {
 // lane g takes entries g, g+G, ..., then a fixed shuffle tree; the launch covers
 // exactly npos * G threads (npos is a multiple of 256), so every lane reaches the
 // shuffles.
-template <class T, int MODE, int G>
-__global__ void __launch_bounds__(BS) k_sell(SellJob<T> j) {
-    pdl_begin();
-    if (j.any && !*j.any) return;
+// AHEAD (launches of a wave or two of blocks, see load_ahead): the row's indices, its
+// diagonal and the first pass of entries are loaded before the wait, and one round of
+// gathers (with b, the row's own value and the flags beside them) leads to the store.
+template <class T, int MODE, int G, bool AHEAD, bool C16>
+__device__ __forceinline__ void sell_rows(const SellJob<T> &j) {
+    pdl_wait_if<!AHEAD>();
+    if (!AHEAD && j.any && !*j.any) return;
     const long long t = (long long)blockIdx.x * BS + threadIdx.x;
     const int q = (int)(t / G), g = (int)(t % G);
     const int r = j.row[q];
     bool ok = r >= 0;
-    if (MODE != SM_RESTRICT && ok && j.active && !j.active[j.rowdir[r]]) ok = false;
-    const int len = ok ? j.len[q] : 0;
+    const int dir = (MODE != SM_RESTRICT && ok && j.active) ? j.rowdir[r] : -1;
+    if (!AHEAD && dir >= 0 && !j.active[dir]) ok = false;
+    int len = ok ? j.len[q] : 0;
     const int base = j.ptr[q >> 5] + (q & 31);
     // the row's own operands are loaded before the dot product (shorter chain); a
-    // restriction row's 16-bit columns are offsets from its coarse point's fine row
+    // restriction row's own operand, and the origin of its 16-bit columns, is its coarse
+    // point's fine row
+    const int rb = (MODE == SM_RESTRICT && ok) ? j.cpts[r] : r;
     T own = T(0), di = T(0), bi = T(0);
-    const int rb = (MODE == SM_RESTRICT && ok && j.col16) ? j.cpts[r] : r;
-    if (ok && g == 0) {
-        if (MODE == SM_RESTRICT) {
-            own = j.in[j.col16 ? rb : j.cpts[r]];
-        } else {
-            own = j.in[r];
-            di = j.dinv[r];
-            bi = j.b[r];
-        }
+    if (!AHEAD && ok && g == 0) {
+        own = j.in[rb];
+        if (MODE != SM_RESTRICT) bi = j.b[r];
     }
+    if (MODE != SM_RESTRICT && ok && g == 0) di = j.dinv[r];
     constexpr int U = sell_unroll<MODE, G>();
-    T acc = j.col16 ? sell_dot16<T, G, U>(base, len, g, rb, j.col16, j.val, j.in)
-                    : sell_dot<T, G, U>(base, len, g, j.col, j.val, j.in);
+    T acc = T(0);
+    int j0 = g;
+    if (AHEAD) {
+        int c[U];
+        T v[U], x[U];
+        sell_load<T, G, U, C16>(base, len, j0, rb, j.col, j.col16, j.val, c, v);
+        pdl_wait_if<AHEAD>();
+        const int any = j.any ? *j.any : 1;
+        const int act = dir >= 0 ? j.active[dir] : 1;
+        if (ok && g == 0) {
+            own = j.in[rb];
+            if (MODE != SM_RESTRICT) bi = j.b[r];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) x[u] = j0 + u * G < len ? j.in[c[u]] : T(0);
+        if (!any) return;
+        ok = ok && act;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (j0 + u * G < len) acc += v[u] * x[u];
+        j0 += U * G;
+    }
+    for (; j0 < len; j0 += U * G) {
+        int c[U];
+        T v[U], x[U];
+        sell_load<T, G, U, C16>(base, len, j0, rb, j.col, j.col16, j.val, c, v);
+#pragma unroll
+        for (int u = 0; u < U; ++u) x[u] = j0 + u * G < len ? j.in[c[u]] : T(0);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (j0 + u * G < len) acc += v[u] * x[u];
+    }
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o, G);
     if (!ok || g != 0) return;
@@ -595,16 +671,22 @@ __global__ void __launch_bounds__(BS) k_sell(SellJob<T> j) {
         j.out[r] = acc + own;
         return;
     }
-    const T v = own + di * (bi - acc);
+    const T vn = own + di * (bi - acc);
     if (MODE == SM_C_FINAL) {
-        if (j.d32) j.d32[r] += (float)v;
-        else j.x64[r] += (double)v;
+        if (j.d32) j.d32[r] += (float)vn;
+        else j.x64[r] += (double)vn;
     } else {
         // the fold's load before the store to out
-        if (MODE == SM_F && j.d32) j.d32[r] += (float)v;
-        else if (MODE == SM_F && j.x64) j.x64[r] += (double)v;
-        j.out[r] = v;
+        if (MODE == SM_F && j.d32) j.d32[r] += (float)vn;
+        else if (MODE == SM_F && j.x64) j.x64[r] += (double)vn;
+        j.out[r] = vn;
     }
+}
+
+template <class T, int MODE, int G, bool AHEAD>
+__global__ void __launch_bounds__(BS) k_sell(SellJob<T> j) {
+    if (j.col16) sell_rows<T, MODE, G, AHEAD, true>(j);
+    else sell_rows<T, MODE, G, AHEAD, false>(j);
 }
 
 // ---- prolongation y = P x_c --------------------------------------------------
@@ -616,12 +698,7 @@ __device__ __forceinline__ void prolong_row(long long i, int8_t c, int p, const 
                                             const T *xc, T *y, T *y2) {
     if (c == CF_COARSEST) return;
     T v = T(0);
-    if (p >= 0) {
-        // both candidates are loaded with the flag (one dependent step, not two)
-        const int8_t cc = cfc[p];
-        const T vf = xcF[p], vc = xc[p];
-        v = cc == CF_F ? vf : vc;
-    }
+    if (p >= 0) v = (cfc[p] == CF_F ? xcF : xc)[p];
     y[i] = v;
     if (y2 && c == CF_C) y2[i] = v;
 }
@@ -631,8 +708,6 @@ __device__ __forceinline__ void prolong_row(long long i, int8_t c, int p, const 
 template <class T>
 __global__ void k_prolong(int n, const int8_t *cf, const int *pmap, const int8_t *cfc, const T *xcF, const T *xc,
                           T *y, T *y2, const int *any) {
-    pdl_begin();
-    if (any && !*any) return;
     const long long i0 = 4LL * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
     if (i0 >= n) return;
     if (i0 + 4 <= n) {
@@ -640,23 +715,27 @@ __global__ void k_prolong(int n, const int8_t *cf, const int *pmap, const int8_t
         const int4 p4 = *reinterpret_cast<const int4 *>(pmap + i0);
         const int8_t c[4] = {(int8_t)c4.x, (int8_t)c4.y, (int8_t)c4.z, (int8_t)c4.w};
         const int p[4] = {p4.x, p4.y, p4.z, p4.w};
-        int8_t cc[4];
-        T vf[4], vc[4];
+        const T *src[4];   // where the coarse value lives: the coarse rows' flags are constants too
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const bool gth = c[u] != CF_COARSEST && p[u] >= 0;
-            cc[u] = gth ? cfc[p[u]] : (int8_t)CF_C;
-            vf[u] = gth ? xcF[p[u]] : T(0);
-            vc[u] = gth ? xc[p[u]] : T(0);
+            src[u] = gth ? (cfc[p[u]] == CF_F ? xcF : xc) + p[u] : nullptr;
         }
+        pdl_wait();
+        const int go = any ? *any : 1;
+        T v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = src[u] ? *src[u] : T(0);
+        if (!go) return;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             if (c[u] == CF_COARSEST) continue;
-            const T v = cc[u] == CF_F ? vf[u] : vc[u];
-            y[i0 + u] = v;
-            if (y2 && c[u] == CF_C) y2[i0 + u] = v;
+            y[i0 + u] = v[u];
+            if (y2 && c[u] == CF_C) y2[i0 + u] = v[u];
         }
     } else {
+        pdl_wait();
+        if (any && !*any) return;
         for (long long i = i0; i < n; ++i) prolong_row<T>(i, cf[i], pmap[i], cfc, xcF, xc, y, y2);
     }
 }
@@ -685,12 +764,15 @@ __global__ void k_fold_coarsest(int n, const T *xco, double *x64, float *d32, fl
 template <class T>
 __global__ void k_jacobi0(int kX, int n, const int *srow, const T *dinv, const T *b, T *x, int zero,
                           const int *any) {
-    pdl_begin();
-    if (any && !*any) return;
     const long long p = kX + (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const int i = srow[p];
-    x[i] = zero ? T(0) : dinv[i] * b[i];
+    const T di = dinv[i];
+    pdl_wait();
+    const int go = any ? *any : 1;
+    const T bi = b[i];
+    if (!go) return;
+    x[i] = zero ? T(0) : di * bi;
 }
 
 // final correction at a CSR level 0: x64 += the coarsest solution on the rows of
@@ -698,12 +780,13 @@ __global__ void k_jacobi0(int kX, int n, const int *srow, const T *dinv, const T
 template <class T>
 __global__ void k_fold_split(int kX, int n, const int *srow, const T *xco, double *x64, float *d32,
                              const int *active, const int *rowdir, float2 *xdd, const int *any) {
-    pdl_begin();
-    if (any && !*any) return;
     int k = kX + blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     int i = srow[k];
-    if (active && !active[rowdir[i]]) return;
+    const int dir = active ? rowdir[i] : 0;
+    pdl_wait();
+    if (any && !*any) return;
+    if (active && !active[dir]) return;
     if (d32) {
         d32[i] += (float)xco[i];
     } else if (xdd) {
@@ -716,34 +799,31 @@ __global__ void k_fold_split(int kX, int n, const int *srow, const T *xco, doubl
 }
 
 // ---- BSR (hex level 0) relaxation, unit diagonal ------------------------------
-template <class T, bool FINAL>
+template <class T, bool FINAL, bool AHEAD>
 __global__ void __launch_bounds__(BS) k_relax_bsr(int n, int N, const int8_t *dsign, const T *vals, const int8_t *cf,
                                                   const T *b, const T *in, T *out, int phase, double *x64,
                                                   const T *xco, const int *active, float2 *xdd) {
-    pdl_begin();
     HexRow q = hex_row(n);
     if (!q.valid) return;
     const long long gi = (long long)q.m * N + 8LL * q.e + q.a;
-    // Loads that decide nothing are issued before any branch: the sweep is latency-
-    // bound, and a load behind a branch on another load costs one more round trip.
-    // The F sweeps (not final) also compute every row's face terms before knowing
-    // whether the row is an F row (a C row's block values are then read for
-    // nothing: a quarter of the rows, against one round trip saved for all).
-    const int act = active ? active[q.m] : 1;
+    // Ahead of the wait the row's kind decides which faces are read; otherwise loads that
+    // decide nothing come before any branch (a load behind a branch on another load costs
+    // one more round trip), and an F sweep reads a C row's faces for nothing.
+    pdl_wait_if<!AHEAD>();
     const int8_t c = cf[gi];
+    const bool mine = c == (phase == 0 ? CF_F : CF_C);
+    const HexFaces<T> fc =
+        hex_faces<T>(n, (long long)N / 8, q.m, q.e, q.a, q.idx, dsign, vals, AHEAD || FINAL ? mine : true);
+    pdl_wait_if<AHEAD>();
+    const int act = active ? active[q.m] : 1;
     const T xin = in[gi], bi = b[gi];
-    T acc = T(0);
-    if (!FINAL)
-        acc = bsr_offdiag<T, T>(n, (long long)N / 8, q.m, q.e, q.a, q.idx, dsign, vals, in + (long long)q.m * N);
+    const T acc = hex_apply<T, T>(fc, in + (long long)q.m * N);
     if (!act) return;
     T v = xin;
     if (c == CF_COARSEST) {   // a matrix whose hierarchy ends at level 0
         if (!FINAL) return;
         v = xco[gi];
-    } else if (c == (phase == 0 ? CF_F : CF_C)) {
-        if (FINAL)
-            acc = bsr_offdiag<T, T>(n, (long long)N / 8, q.m, q.e, q.a, q.idx, dsign, vals,
-                                    in + (long long)q.m * N);
+    } else if (mine) {
         v = v + (bi - (acc + v));
     }
     if (!FINAL) {
@@ -776,13 +856,13 @@ __device__ __forceinline__ void x_add(long long gi, float v, float *d32, float2 
 
 // rows at split positions [k0, k0 + cnt): F sweep (out, optional fold into x) or the
 // final C sweep (into x)
-template <bool FINAL>
+template <bool FINAL, bool AHEAD>
 __global__ void __launch_bounds__(BS) k_relax0_split(int n, int N, const int8_t *dsign, const int *srow, int k0,
                                                      int cnt, const float4 *v0, const float *b, const float *in,
                                                      float *out, bool fold, float *d32, float2 *xdd, double *x64,
                                                      const int *active, const int *any) {
-    pdl_begin();
-    if (any && !*any) return;
+    pdl_wait_if<!AHEAD>();
+    if (!AHEAD && any && !*any) return;
     const int k = blockIdx.x * BS + threadIdx.x;
     if (k >= cnt) return;
     const int gi = srow[k0 + k];
@@ -792,25 +872,32 @@ __global__ void __launch_bounds__(BS) k_relax0_split(int n, int N, const int8_t 
     const int ix = e % n, t = e / n, iy = t % n, iz = t / n;
     const int idx[3] = {ix, iy, iz};
     const int stride[3] = {1, n, n * n};
-    const int act = active ? active[m] : 1;
-    const float xin = in[gi], bi = b[gi];
     const float *xm = in + (long long)m * N;
-    float acc = 0.0f;
+    int act = 1;
+    float xin = 0.0f, bi = 0.0f, acc = 0.0f;
+    if (!AHEAD) {
+        act = active ? active[m] : 1;
+        xin = in[gi];
+        bi = b[gi];
+    }
+    HexFaces<float> fc;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         const int sg = dsign[3 * m + d];
-        if (sg == 0) continue;
-        const bool has = sg > 0 ? idx[d] > 0 : idx[d] < n - 1;
-        if (!has) continue;
-        const int ep = sg > 0 ? e - stride[d] : e + stride[d];
-        const int o = sg > 0 ? 1 : 0;
-        const float4 w = __ldcs(v0 + 3LL * (k0 + k) + d);
-        const float *xb = xm + 8LL * ep;
-        acc += w.x * xb[face_node(d, o, 0)];
-        acc += w.y * xb[face_node(d, o, 1)];
-        acc += w.z * xb[face_node(d, o, 2)];
-        acc += w.w * xb[face_node(d, o, 3)];
+        const bool has = sg > 0 ? idx[d] > 0 : (sg < 0 && idx[d] < n - 1);
+        fc.off[d] = has ? 8 * (sg > 0 ? e - stride[d] : e + stride[d]) : -1;
+        fc.o[d] = sg > 0 ? 1 : 0;
+        const float4 w = has ? __ldcs(v0 + 3LL * (k0 + k) + d) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        fc.w[d] = {w.x, w.y, w.z, w.w};
     }
+    if (AHEAD) {
+        pdl_wait_if<AHEAD>();
+        if (any && !*any) return;
+        act = active ? active[m] : 1;
+        xin = in[gi];
+        bi = b[gi];
+    }
+    acc = hex_apply<float, float>(fc, xm);
     if (!act) return;
     const float v = xin + (bi - (acc + xin));
     if (!FINAL) {
@@ -922,8 +1009,22 @@ template <>
 const float *lv_dinv<float>(const Level &L) { return L.dinv32; }
 template <>
 const double *lv_dinv<double>(const Level &L) { return L.dinv; }
+// Loads ahead of the wait pay on launches whose blocks are resident in a wave or two: there
+// the chain of dependent loads is the kernel's time (and the registers that hold the
+// entries cost nothing).  On larger ones most blocks start after the wait anyway, and the
+// registers and the delayed vector loads cost resident warps.  Solves by blocks per SM up
+// to which kernels load ahead (0: none, 1000: all):
+//                              0        6       12     1000
+//   13^3 S4 host            56.7 ms  54.2 ms  50.5 ms  52.3 ms
+//   16^3 x 6 tets S4       136.6    134.1    129.3    126.5
+//   24^3 x 4, one solve      4.23     3.63     3.64     3.70
+//   24^3 S4 gradient       328.8    317.0    314.8    319.9
+//   32^3 S4                179.6    181.3    180.1    193.5
+constexpr int AHEAD_BLOCKS_PER_SM = 12;
+bool load_ahead(long long blocks, int sms) { return blocks <= (long long)AHEAD_BLOCKS_PER_SM * sms; }
+
 template <class T, int MODE>
-void launch_sell_g(const Sell &S, SellJob<T> j, int G, cudaStream_t s) {
+void launch_sell_g(const Sell &S, SellJob<T> j, int G, int sms, cudaStream_t s) {
     j.npos = S.npos;
     j.ptr = S.ptr;
     j.row = S.row;
@@ -931,11 +1032,13 @@ void launch_sell_g(const Sell &S, SellJob<T> j, int G, cudaStream_t s) {
     j.col = S.col;
     j.col16 = S.col16;
     j.val = (const T *)S.val;
+    const unsigned nb = blocks_for((long long)G * S.npos, BS);
+    auto go = [&](auto ahead, auto plain) { launch_pdl(load_ahead(nb, sms) ? ahead : plain, nb, BS, s, j); };
     switch (G) {
-        case 1: launch_pdl(k_sell<T, MODE, 1>, blocks_for(S.npos, BS), BS, s, j); break;
-        case 2: launch_pdl(k_sell<T, MODE, 2>, blocks_for(2LL * S.npos, BS), BS, s, j); break;
-        case 4: launch_pdl(k_sell<T, MODE, 4>, blocks_for(4LL * S.npos, BS), BS, s, j); break;
-        default: launch_pdl(k_sell<T, MODE, 8>, blocks_for(8LL * S.npos, BS), BS, s, j); break;
+        case 1: go(k_sell<T, MODE, 1, true>, k_sell<T, MODE, 1, false>); break;
+        case 2: go(k_sell<T, MODE, 2, true>, k_sell<T, MODE, 2, false>); break;
+        case 4: go(k_sell<T, MODE, 4, true>, k_sell<T, MODE, 4, false>); break;
+        default: go(k_sell<T, MODE, 8, true>, k_sell<T, MODE, 8, false>); break;
     }
     PR_LAUNCH();
 }
@@ -953,7 +1056,7 @@ int sell_lanes(const Sell &S, int sms) {
 template <class T, int MODE>
 void launch_sell(const Sell &S, SellJob<T> j, int sms, cudaStream_t s) {
     if (S.nrows <= 0) return;
-    launch_sell_g<T, MODE>(S, j, sell_lanes(S, sms), s);
+    launch_sell_g<T, MODE>(S, j, sell_lanes(S, sms), sms, s);
 }
 
 // F sweep over the F rows (fold: x64 += the new values, the last level-0 sweep)
@@ -1094,13 +1197,17 @@ void vcycle_t(Hier &h, double *x64, float *d32, const int *active, ProfSlot *ps)
             if (prof) { rec_event(ps->relax0[0], s); ps->relax_timed = true; }
             for (int f = 0; f < fs; ++f, cur ^= 1)
                 if (L.nF > 0) {
-                    launch_pdl(k_relax0_split<false>, blocks_for(L.nF, BS), BS, s, h.hex_n, N, h.dsign, L.srow, 0,
+                    launch_pdl(load_ahead(blocks_for(L.nF, BS), h.sms) ? k_relax0_split<false, true>
+                                                                       : k_relax0_split<false, false>,
+                               blocks_for(L.nF, BS), BS, s, h.hex_n, N, h.dsign, L.srow, 0,
                                L.nF, h.v0, (const float *)L.vb, (const float *)bufs[cur], (float *)bufs[cur ^ 1],
                                f == fs - 1, d32, xdd, x64, active, any);
                     PR_LAUNCH();
                 }
             if (L.nC > 0) {
-                launch_pdl(k_relax0_split<true>, blocks_for(L.nC, BS), BS, s, h.hex_n, N, h.dsign, L.srow, L.nF,
+                launch_pdl(load_ahead(blocks_for(L.nC, BS), h.sms) ? k_relax0_split<true, true>
+                                                                   : k_relax0_split<true, false>,
+                           blocks_for(L.nC, BS), BS, s, h.hex_n, N, h.dsign, L.srow, L.nF,
                            L.nC, h.v0, (const float *)L.vb, (const float *)bufs[cur], (float *)nullptr, true, d32,
                            xdd, x64, active, any);
                 PR_LAUNCH();
@@ -1115,13 +1222,14 @@ void vcycle_t(Hier &h, double *x64, float *d32, const int *active, ProfSlot *ps)
             int N = h.n0[0];
             dim3 grid(blocks_for(h.hex_n, 32), h.hex_n * h.hex_n, h.ndir);
             const T *vals = std::is_same<T, float>::value ? (const T *)h.bsr32 : (const T *)h.bsr64;
+            const bool ah = load_ahead((long long)grid.x * grid.y * grid.z, h.sms);
             if (prof) { rec_event(ps->relax0[0], s); ps->relax_timed = true; }
             for (int f = 0; f < fs; ++f, cur ^= 1) {
-                launch_pdl(k_relax_bsr<T, false>, grid, BS, s, h.hex_n, N, h.dsign, vals, L.cf, (const T *)L.vb, bufs[cur],
+                launch_pdl(ah ? k_relax_bsr<T, false, true> : k_relax_bsr<T, false, false>, grid, BS, s, h.hex_n, N, h.dsign, vals, L.cf, (const T *)L.vb, bufs[cur],
                                                           bufs[cur ^ 1], 0, nullptr, nullptr, active, nullptr);
                 PR_LAUNCH();
             }
-            launch_pdl(k_relax_bsr<T, true>, grid, BS, s, h.hex_n, N, h.dsign, vals, L.cf, (const T *)L.vb, bufs[cur],
+            launch_pdl(ah ? k_relax_bsr<T, true, true> : k_relax_bsr<T, true, false>, grid, BS, s, h.hex_n, N, h.dsign, vals, L.cf, (const T *)L.vb, bufs[cur],
                                                      nullptr, 1, x64, (const T *)L.vx, active, xdd);
             PR_LAUNCH();
             if (prof) rec_event(ps->relax0[1], s);
@@ -1401,27 +1509,28 @@ void residual0_launch(Hier &h, const double *b, const double *x, const int *act,
     Level &L = h.lev[0];
     dim3 grid(h.maxblk, h.ndir);
     bool f32 = h.prm.precision >= 1;
+    const int N = h.n0[0];
+    const dim3 g3(blocks_for(h.hex_n, 32), h.hex_n * h.hex_n, h.ndir);
+    const bool ah3 = load_ahead((long long)g3.x * g3.y * g3.z, h.sms);
+    const bool ah = load_ahead((long long)grid.x * grid.y, h.sms);
     if (h.bsr0 && h.dd) {
-        int N = h.n0[0];
-        dim3 g3(blocks_for(h.hex_n, 32), h.hex_n * h.hex_n, h.ndir);
-        launch_pdl(k_res0_bsr_dd, g3, BS, s, h.hex_n, N, h.dsign, h.bsr_dd, h.b_dd, h.x_dd, (float *)L.vb, r2,
-                   h.partials, h.maxblk, act);
+        launch_pdl(ah3 ? k_res0_bsr_dd<true> : k_res0_bsr_dd<false>, g3, BS, s, h.hex_n, N, h.dsign, h.bsr_dd, h.b_dd,
+                   h.x_dd, (float *)L.vb, r2, h.partials, h.maxblk, act);
     } else if (h.bsr0) {
-        int N = h.n0[0];
-        dim3 g3(blocks_for(h.hex_n, 32), h.hex_n * h.hex_n, h.ndir);
         if (f32)
-            launch_pdl(k_res0_bsr<float>, g3, BS, s, h.hex_n, N, h.dsign, h.bsr64, b, x, (float *)L.vb, r2,
-                       h.partials, h.maxblk, act, zero_x ? 1 : 0);
+            launch_pdl(ah3 ? k_res0_bsr<float, true> : k_res0_bsr<float, false>, g3, BS, s, h.hex_n, N, h.dsign, h.bsr64,
+                       b, x, (float *)L.vb, r2, h.partials, h.maxblk, act, zero_x ? 1 : 0);
         else
-            launch_pdl(k_res0_bsr<double>, g3, BS, s, h.hex_n, N, h.dsign, h.bsr64, b, x, (double *)L.vb,
-                       (float *)nullptr, h.partials, h.maxblk, act, zero_x ? 1 : 0);
+            launch_pdl(ah3 ? k_res0_bsr<double, true> : k_res0_bsr<double, false>, g3, BS, s, h.hex_n, N, h.dsign,
+                       h.bsr64, b, x, (double *)L.vb, (float *)nullptr, h.partials, h.maxblk, act, zero_x ? 1 : 0);
     } else {
         if (f32)
-            launch_pdl(k_res0_csr<float>, grid, BS, s, h.d_row00, h.d_n0, L.rowptr, L.col, L.val, b, x, (float *)L.vb,
-                       r2, h.partials, h.maxblk, act, zero_x ? 1 : 0);
+            launch_pdl(ah ? k_res0_csr<float, true> : k_res0_csr<float, false>, grid, BS, s, h.d_row00, h.d_n0,
+                       L.rowptr, L.col, L.val, b, x, (float *)L.vb, r2, h.partials, h.maxblk, act, zero_x ? 1 : 0);
         else
-            launch_pdl(k_res0_csr<double>, grid, BS, s, h.d_row00, h.d_n0, L.rowptr, L.col, L.val, b, x,
-                       (double *)L.vb, (float *)nullptr, h.partials, h.maxblk, act, zero_x ? 1 : 0);
+            launch_pdl(ah ? k_res0_csr<double, true> : k_res0_csr<double, false>, grid, BS, s, h.d_row00, h.d_n0,
+                       L.rowptr, L.col, L.val, b, x, (double *)L.vb, (float *)nullptr, h.partials, h.maxblk, act,
+                       zero_x ? 1 : 0);
     }
     PR_LAUNCH();
 }
@@ -1509,7 +1618,7 @@ std::mutex g_tune_mutex;
 std::map<std::tuple<int, int, int, long long>, int> g_tune;
 
 template <class T, int MODE>
-void tune_store(Sell &S, const SellJob<T> &j, cudaStream_t s, cudaEvent_t e0, cudaEvent_t e1) {
+void tune_store(Sell &S, const SellJob<T> &j, int sms, cudaStream_t s, cudaEvent_t e0, cudaEvent_t e1) {
     if (S.nrows <= 0) return;
     const auto key = std::make_tuple(MODE, (int)sizeof(T), S.npos, S.nnz);
     // held while tuning: hierarchies set up at the same time on other threads (the
@@ -1521,9 +1630,9 @@ void tune_store(Sell &S, const SellJob<T> &j, cudaStream_t s, cudaEvent_t e0, cu
     int best = 1;
     float tbest = 0;
     for (int G = 1; G <= 8; G *= 2) {
-        launch_sell_g<T, MODE>(S, j, G, s);
+        launch_sell_g<T, MODE>(S, j, G, sms, s);
         PR_CUDA(cudaEventRecord(e0, s));
-        for (int r = 0; r < 3; ++r) launch_sell_g<T, MODE>(S, j, G, s);
+        for (int r = 0; r < 3; ++r) launch_sell_g<T, MODE>(S, j, G, sms, s);
         PR_CUDA(cudaEventRecord(e1, s));
         PR_CUDA(cudaEventSynchronize(e1));
         float ms = 0;
@@ -1553,15 +1662,15 @@ void autotune_t(Hier &h) {
         j.b = (const T *)L.vb;
         j.out = (T *)L.vxn;
         j.rowdir = L.rowdir;
-        tune_store<T, SM_F>(L.sF, j, s, e0, e1);
-        tune_store<T, SM_C>(L.sC, j, s, e0, e1);
-        tune_store<T, SM_F>(L.sX, j, s, e0, e1);
+        tune_store<T, SM_F>(L.sF, j, h.sms, s, e0, e1);
+        tune_store<T, SM_C>(L.sC, j, h.sms, s, e0, e1);
+        tune_store<T, SM_F>(L.sX, j, h.sms, s, e0, e1);
         if (l + 1 < NL && L.sZ.nrows > 0) {
             SellJob<T> r{};
             r.in = (const T *)L.vb;
             r.out = (T *)h.lev[l + 1].vb;
             r.cpts = L.cpts;
-            tune_store<T, SM_RESTRICT>(L.sZ, r, s, e0, e1);
+            tune_store<T, SM_RESTRICT>(L.sZ, r, h.sms, s, e0, e1);
         }
     }
     // the tuning launches wrote only the zeroed work vectors: clear them again
@@ -1628,11 +1737,11 @@ void inner_cycle(Hier &h, ProfSlot *ps) {
     Level &L = h.lev[0];
     if (h.bsr0) {
         dim3 g3(blocks_for(h.hex_n, 32), h.hex_n * h.hex_n, h.ndir);
-        launch_pdl(k_res32_bsr, g3, BS, s, h.hex_n, h.n0[0], h.dsign, (const float *)h.bsr32, (const float *)h.r32,
+        launch_pdl(load_ahead((long long)g3.x * g3.y * g3.z, h.sms) ? k_res32_bsr<true> : k_res32_bsr<false>, g3, BS, s, h.hex_n, h.n0[0], h.dsign, (const float *)h.bsr32, (const float *)h.r32,
                    (const float *)h.d32, (float *)L.vb, h.partials, h.maxblk, (const int *)h.iactive);
     } else {
         dim3 grid(h.maxblk, h.ndir);
-        launch_pdl(k_res32_csr, grid, BS, s, (const int *)h.d_row00, (const int *)h.d_n0, (const int *)L.rowptr,
+        launch_pdl(load_ahead((long long)grid.x * grid.y, h.sms) ? k_res32_csr<true> : k_res32_csr<false>, grid, BS, s, (const int *)h.d_row00, (const int *)h.d_n0, (const int *)L.rowptr,
                    (const int *)L.col, (const float *)h.val32, (const float *)h.r32, (const float *)h.d32,
                    (float *)L.vb, h.partials, h.maxblk, (const int *)h.iactive);
     }
