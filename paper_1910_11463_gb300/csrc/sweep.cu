@@ -27,7 +27,6 @@ __device__ __forceinline__ int sw_face_node(int d, int o, int t) {
 
 __global__ void __launch_bounds__(SW_BS) k_sweep_wave(int n, int N, int wave, const int8_t *dsign,
                                                       const double *bsr64, const double *b, double *x) {
-    pdl_begin();
     const int m = blockIdx.y;
     const long long t = (long long)blockIdx.x * SW_BS + threadIdx.x;
     const long long pair = t >> 3;
@@ -44,18 +43,25 @@ __global__ void __launch_bounds__(SW_BS) k_sweep_wave(int n, int N, int wave, co
     const int e = idx[0] + n * (idx[1] + n * idx[2]);
     const double *base = bsr64 + (((long long)m * E + e) * 3) * 32 + a * 4;
     const double *xm = x + (long long)m * N;
+    // face rows before the wait for the previous wavefront (constants of the solve)
+    double w[3][4];
+    int off[3], o[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const bool has = sg[d] > 0 ? idx[d] > 0 : (sg[d] < 0 && idx[d] < n - 1);
+        off[d] = has ? 8 * (sg[d] > 0 ? e - stride[d] : e + stride[d]) : -1;
+        o[d] = sg[d] > 0 ? 1 : 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[d][k] = has ? base[d * 32 + k] : 0.0;
+    }
+    pdl_wait();
     double acc = 0.0;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        if (sg[d] == 0) continue;
-        const bool has = sg[d] > 0 ? idx[d] > 0 : idx[d] < n - 1;
-        if (!has) continue;
-        const int ep = sg[d] > 0 ? e - stride[d] : e + stride[d];
-        const int o = sg[d] > 0 ? 1 : 0;
-        const double *w = base + d * 32;
-        const double *xb = xm + 8LL * ep;
+        if (off[d] < 0) continue;
+        const double *xb = xm + off[d];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) acc += w[k] * xb[sw_face_node(d, o, k)];
+        for (int k = 0; k < 4; ++k) acc += w[d][k] * xb[sw_face_node(d, o[d], k)];
     }
     const long long gi = (long long)m * N + 8LL * e + a;
     x[gi] = b[gi] - acc;

@@ -171,21 +171,42 @@ __global__ void k_sd_scatter(long long Eb, const int *level, const int8_t *role,
 }
 
 // one level's single elements: x_r = b_r - sum over the row's upwind entries
-// (stored order; this file is compiled without contraction into FMA)
-__global__ void __launch_bounds__(SD_BS) k_sd_level(int nb, const int *list, int count, const int *rowptr,
-                                                    const int *col, const double *val, const double *b, double *x) {
-    pdl_begin();
+// (stored order; this file is compiled without contraction into FMA).  A solve is a chain
+// of one such launch per level, a few thousand rows each, so its time is the dependent
+// loads of a row: the element, its row's extent and up to SD_U entries (a P1 row holds at
+// most 13) are loaded before the wait for the previous level, and only the gathers of
+// upwind values, the sum and the store follow it.
+constexpr int SD_U = 13;
+template <int NB>
+__global__ void __launch_bounds__(SD_BS) k_sd_level(const int *list, int count, const int *rowptr, const int *col,
+                                                    const double *val, const double *b, double *x) {
     const long long t = (long long)blockIdx.x * SD_BS + threadIdx.x;
-    const long long i = t / nb;
+    const long long i = t / NB;
     if (i >= count) return;
-    const int a = (int)(t - i * nb);
-    const long long g = list[i];
-    const long long r = g * nb + a;
-    double s = b[r];
-    for (int p = rowptr[r]; p < rowptr[r + 1]; ++p) {
-        const int c = col[p];
-        if (c / nb == g) continue;
-        s = s - val[p] * x[c];
+    const int a = (int)(t - i * NB);
+    const int g = list[i];
+    const long long r = (long long)g * NB + a;
+    const int p1 = rowptr[r + 1];
+    int p = rowptr[r];
+    int c[SD_U];
+    double v[SD_U];
+#pragma unroll
+    for (int u = 0; u < SD_U; ++u) {
+        c[u] = p + u < p1 ? col[p + u] : -1;
+        v[u] = p + u < p1 ? val[p + u] : 0.0;
+        if (c[u] / NB == g) c[u] = -1;   // the element's own entries (identity block)
+    }
+    pdl_wait();
+    double s = b[r], xs[SD_U];
+#pragma unroll
+    for (int u = 0; u < SD_U; ++u) xs[u] = c[u] >= 0 ? x[c[u]] : 0.0;
+#pragma unroll
+    for (int u = 0; u < SD_U; ++u)
+        if (c[u] >= 0) s = s - v[u] * xs[u];
+    for (p += SD_U; p < p1; ++p) {
+        const int cc = col[p];
+        if (cc / NB == g) continue;
+        s = s - val[p] * x[cc];
     }
     x[r] = s;
 }
@@ -417,7 +438,7 @@ void sweep_plan_launch(const SweepPlan &P, const int *rowptr, const int *col, co
     for (int l = 0; l < P.nlev; ++l) {
         const long long c = P.off[l + 1] - P.off[l];
         if (c > 0) {
-            launch_pdl(k_sd_level, dim3(blocks_for(c * P.nb, SD_BS)), dim3(SD_BS), s, P.nb,
+            launch_pdl(P.nb == 4 ? k_sd_level<4> : k_sd_level<8>, dim3(blocks_for(c * P.nb, SD_BS)), dim3(SD_BS), s,
                        (const int *)(P.list + P.off[l]), (int)c, rowptr, col, val, b, x);
             PR_LAUNCH();
         }
