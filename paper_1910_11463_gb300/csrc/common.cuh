@@ -180,6 +180,11 @@ struct Level {
     int *srow = nullptr, *sptr = nullptr, *scol = nullptr;
     void *sval = nullptr;
     int *d_cseg_s0 = nullptr;
+    // dense form of the coarsest sweeps (segments of at most CD_MAX rows): the matrix that
+    // takes b to the result of the sweeps, per segment, in the order the kernel reads it
+    void *cB = nullptr;
+    int *d_cB_off = nullptr;   // first value of each segment, in units of CD_ROWS values
+    int cseg_max = 0;          // rows of the largest segment
     Sell sF, sC, sZ, sX;
     // V-cycle work vectors (precision of the hierarchy); vF is the buffer (vy or vxn)
     // that holds the F rows after the last F sweep, C rows are then in vx
@@ -196,6 +201,9 @@ constexpr int SD_MAXE = 8;
 // entries (value + column), four vectors and row pointer fit is swept in shared
 // memory; a level with a larger one gets a SELL copy of its coarsest rows instead.
 constexpr int CS_SMEM = 40 * 1024;
+// Coarsest segments of at most CD_MAX rows (the library's max_coarse is 100) apply their
+// sweeps as one dense product, CD_ROWS rows to a block.
+constexpr int CD_MAX = 128, CD_ROWS = 32;
 struct SweepPlan {
     int nb = 0, nlev = 0, ncomp = 0;
     int *list = nullptr;                     // single elements, level by level
@@ -348,6 +356,7 @@ void inner_cycle(Hier &h, ProfSlot *ps);
 void fold_delta(Hier &h, double *x);
 // double-float mode (h.dd): b and x to pairs before a solve, x back after it; the
 // residual and the final relaxation then work on h.b_dd / h.x_dd
+void coarsest_dense(Hier &h, Level &L);   // cB of a level whose segments are all small
 void dd_enable(Hier &h);            // bsr_dd from bsr64 (frees bsr64), vectors
 void split0_enable(Hier &h);        // v0 from bsr32 (frees bsr32)
 void dd_load(Hier &h, const double *b, const double *x);

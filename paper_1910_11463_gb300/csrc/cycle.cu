@@ -1003,6 +1003,80 @@ __global__ void k_coarsest(const int *seg_row0, const int *seg_n, const int *seg
                     sweeps, cs_sm, &cs_bad);
 }
 
+// ---- coarsest level: the sweeps as one dense product ----------------------------------
+// The coarse_sweeps Jacobi sweeps from zero are linear in b: x = B b with
+// B = sum_{k < sweeps} (I - D^{-1} A)^k D^{-1}, an nr x nr matrix of a segment of nr rows.
+// The sweeps of a 100-row segment are a chain of 20 steps in one CTA, each a row's
+// dependent loads and FP64 (or FP32) adds and a barrier: 56 us in FP64, 14-17 us in FP32,
+// the longest kernel of a small mesh's V-cycle.  B is formed once per setup in FP64 (by
+// sweeping the unit vectors) and kept in the cycle precision; its product reads it before
+// the wait for the restriction, so 4 lanes a row are left with nr / 4 multiply-adds.  8^3
+// S2 in FP64 26.7 -> 20.7 ms, 13^3 S4 50.5 -> 48.0, 7^3 tet FP64 gradient 131 -> 105.
+// Segments past CD_MAX rows keep the sweeps (B grows with nr^2).
+template <class T>
+__global__ void __launch_bounds__(4 * CD_ROWS) k_coarsest_dense(const int *seg_row0, const int *seg_n, const int *off,
+                                                                const T *B, const T *b, T *x, const int *any) {
+    constexpr int NT = 4 * CD_ROWS, NI = CD_MAX / 4;
+    __shared__ T sb[CD_MAX];
+    const int sg = blockIdx.x, r0 = seg_row0[sg], nr = seg_n[sg];
+    if ((int)blockIdx.y * CD_ROWS >= nr) return;
+    const int ni = (nr + 3) / 4, t = threadIdx.x, q = t & 3;
+    const T *Bt = B + (long long)off[sg] * CD_ROWS + (long long)blockIdx.y * NT * ni + t;
+    T w[NI];
+#pragma unroll
+    for (int i = 0; i < NI; ++i) w[i] = i < ni ? Bt[i * NT] : T(0);
+    pdl_wait();
+    const int go = any ? *any : 1;
+    sb[t] = t < nr ? b[r0 + t] : T(0);
+    if (!go) return;
+    __syncthreads();
+    T acc = T(0);
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+        if (i < ni) acc += w[i] * sb[4 * i + q];
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+    const int r = blockIdx.y * CD_ROWS + (t >> 2);
+    if (q == 0 && r < nr) x[r0 + r] = acc;
+}
+static_assert(4 * CD_ROWS == CD_MAX, "one right-hand side value per thread");
+
+// CD_COLS columns of B per block: the sweeps on their unit vectors in shared memory
+constexpr int CD_COLS = 8;
+template <class T>
+__global__ void __launch_bounds__(256) k_coarsest_form(const int *seg_row0, const int *seg_n, const int *off,
+                                                       const int *rowptr, const int *col, const double *val,
+                                                       const double *dinv, int sweeps, T *B) {
+    __shared__ double X[2][CD_MAX][CD_COLS];
+    const int sg = blockIdx.x, r0 = seg_row0[sg], nr = seg_n[sg], c0 = blockIdx.y * CD_COLS;
+    if (c0 >= nr) return;
+    for (int e = threadIdx.x; e < nr * CD_COLS; e += 256) X[0][e / CD_COLS][e % CD_COLS] = 0.0;
+    __syncthreads();
+    int cur = 0;
+    for (int s = 0; s < sweeps; ++s, cur ^= 1) {
+        for (int e = threadIdx.x; e < nr * CD_COLS; e += 256) {
+            const int i = e / CD_COLS, c = e % CD_COLS;
+            double acc = 0.0;
+            for (int p = rowptr[r0 + i]; p < rowptr[r0 + i + 1]; ++p) {
+                const int j = col[p] - r0;
+                if (j >= 0 && j < nr) acc += val[p] * X[cur][j][c];
+            }
+            X[cur ^ 1][i][c] = X[cur][i][c] + dinv[r0 + i] * ((c0 + c == i ? 1.0 : 0.0) - acc);
+        }
+        __syncthreads();
+    }
+    // value (row, column j) in k_coarsest_dense's order: row block, j / 4, row in the
+    // block, j % 4
+    const int ni = (nr + 3) / 4;
+    T *Bs = B + (long long)off[sg] * CD_ROWS;
+    for (int e = threadIdx.x; e < nr * CD_COLS; e += 256) {
+        const int i = e / CD_COLS, j = c0 + e % CD_COLS;
+        if (j < nr)
+            Bs[(long long)(i / CD_ROWS) * 4 * CD_ROWS * ni + (j / 4) * 4 * CD_ROWS + (i % CD_ROWS) * 4 + j % 4] =
+                (T)X[cur][i][e % CD_COLS];
+    }
+}
+
 template <class T>
 const T *lv_dinv(const Level &L);
 template <>
@@ -1166,6 +1240,11 @@ void vcycle_t(Hier &h, double *x64, float *d32, const int *active, ProfSlot *ps)
             if (tx) rec_event(ps->lvx[2 * l], s);
             coarsest_sell<T>(L, h.prm.coarse_sweeps, any, h.sms, s);
             if (tx) rec_event(ps->lvx[2 * l + 1], s);
+        } else if (L.n_cseg && L.cB) {
+            launch_pdl(k_coarsest_dense<T>, dim3(L.n_cseg, (L.cseg_max + CD_ROWS - 1) / CD_ROWS), dim3(4 * CD_ROWS), s,
+                       (const int *)L.d_cseg_row0, (const int *)L.d_cseg_n, (const int *)L.d_cB_off, (const T *)L.cB,
+                       (const T *)L.vb, (T *)L.vx, any);
+            PR_LAUNCH();
         } else if (L.n_cseg) {
             launch_pdl(k_coarsest<T>, L.n_cseg, 256, s, L.d_cseg_row0, L.d_cseg_n, L.d_cseg_s0, L.sptr, L.scol,
                                                    (const T *)L.sval, lv_dinv<T>(L), (const T *)L.vb, (T *)L.vx,
@@ -1259,6 +1338,36 @@ void vcycle_t(Hier &h, double *x64, float *d32, const int *active, ProfSlot *ps)
 }
 
 }  // namespace
+
+void coarsest_dense(Hier &h, Level &L) {
+    cudaStream_t s = h.stream;
+    std::vector<int> off;
+    long long at = 0;   // in units of CD_ROWS values: a row block holds 4 * ceil(nr / 4) of them
+    int mx = 0;
+    for (int d = 0; d < h.ndir; ++d)
+        if (L.nrows[d] > 0 && L.coarsest[d]) {
+            const int nr = L.nrows[d];
+            mx = std::max(mx, nr);
+            if (mx > CD_MAX || at > 0x7fffffffLL) return;
+            off.push_back((int)at);
+            at += (long long)((nr + CD_ROWS - 1) / CD_ROWS) * 4 * ((nr + 3) / 4);
+        }
+    const size_t es = h.prm.precision >= 1 ? sizeof(float) : sizeof(double);
+    L.cseg_max = mx;
+    L.cB = dmalloc<char>((size_t)at * CD_ROWS * es, s);
+    PR_CUDA(cudaMemsetAsync(L.cB, 0, (size_t)at * CD_ROWS * es, s));   // the columns past nr of a row's last four
+    L.d_cB_off = dmalloc<int>(off.size(), s);
+    PR_CUDA(cudaMemcpyAsync(L.d_cB_off, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice, s));
+    const dim3 grid(L.n_cseg, (mx + CD_COLS - 1) / CD_COLS);
+    if (h.prm.precision >= 1)
+        k_coarsest_form<float><<<grid, 256, 0, s>>>(L.d_cseg_row0, L.d_cseg_n, L.d_cB_off, L.rowptr, L.col, L.val,
+                                                    L.dinv, h.prm.coarse_sweeps, (float *)L.cB);
+    else
+        k_coarsest_form<double><<<grid, 256, 0, s>>>(L.d_cseg_row0, L.d_cseg_n, L.d_cB_off, L.rowptr, L.col, L.val,
+                                                     L.dinv, h.prm.coarse_sweeps, (double *)L.cB);
+    PR_LAUNCH();
+    PR_CUDA(cudaStreamSynchronize(s));   // 'off' is pageable host memory
+}
 
 void alloc_cycle_vectors(Hier &h) {
     size_t es = h.prm.precision >= 1 ? sizeof(float) : sizeof(double);

@@ -1520,7 +1520,7 @@ void build_split(Hier &h, Level &L, bool with_fc) {
 void free_level(Level &L, cudaStream_t s) {
     void *ptrs[] = {L.rowptr, L.col, L.val, L.dinv, L.dinv32, L.cf, L.pmap, L.rowdir, L.cpts,
                     L.zrowptr, L.zcol, L.zval, L.d_row0, L.d_cseg_row0, L.d_cseg_n,
-                    L.srow, L.sptr, L.scol, L.sval, L.d_cseg_s0,
+                    L.srow, L.sptr, L.scol, L.sval, L.d_cseg_s0, L.cB, L.d_cB_off,
                     L.sF.ptr, L.sF.row, L.sF.len, L.sF.col, L.sF.col16, L.sF.val, L.sC.ptr, L.sC.row, L.sC.len,
                     L.sC.col, L.sC.col16, L.sC.val, L.sZ.ptr, L.sZ.row, L.sZ.len, L.sZ.col, L.sZ.col16, L.sZ.val,
                     L.sX.ptr, L.sX.row, L.sX.len, L.sX.col, L.sX.col16, L.sX.val, L.vb, L.vx, L.vxn, L.vy};
@@ -1952,6 +1952,7 @@ void build_hierarchy(Hier &h) {
     for (size_t l = 0; l < h.lev.size(); ++l) {
         Level &L = h.lev[l];
         build_split(h, L, !(l == 0 && h.bsr0));
+        if (L.n_cseg && L.sX.nrows == 0) coarsest_dense(h, L);
         if (L.nc > 0) {
             build_sell(h, L.sZ, nullptr, L.nc, L.zrowptr, L.zcol, L.zval);
             sell_compress_cols(h, L.sZ, L.cpts);   // offsets from each coarse point's fine row

@@ -35,3 +35,30 @@ def test_batch_size_does_not_change_the_flux(pair, mesh, n, precision, inner_tol
         assert info["batches"] == (1 if batch == 0 else prob.M)
         out.append(phi.cpu().numpy())
     assert np.linalg.norm(out[0] - out[1]) <= tol * np.linalg.norm(out[0])
+
+
+# the coarsest sweeps as a dense product against plain sweeps: segments of one row, of
+# a row block and its neighbours, the largest, and one past it (which keeps the sweeps); the
+# two differ by the rounding of a few dozen additions
+@pytest.mark.parametrize("n", [1, 3, 31, 32, 33, 97, 128, 129])
+@pytest.mark.parametrize("sweeps", [0, 1, 7])
+def test_coarsest_product_equals_sweeps(pair, n, sweeps):
+    g = np.random.default_rng(n)
+    A = np.eye(n) + np.tril(g.uniform(-1, 1, (n, n)) * (g.random((n, n)) < 0.2), -1) / np.sqrt(n)
+    A[np.arange(n), np.arange(n)] += 0.5 * g.random(n)
+    ci = [np.nonzero(r)[0] for r in A]
+    rp = np.concatenate([[0], np.cumsum([len(c) for c in ci])]).astype(np.int32)
+    col = np.concatenate(ci).astype(np.int32)
+    val = np.concatenate([A[i, c] for i, c in enumerate(ci)])
+    b = g.standard_normal(n)
+    want = np.zeros(n)
+    for _ in range(sweeps):
+        want = want + (b - A @ want) / np.diag(A)
+    for precision, tol in ((0, 1e-13), (1, 2e-6)):
+        dev = [torch.as_tensor(a, device="cuda") for a in (rp, col, val)]
+        h = pair.Hierarchy([tuple(dev)] * 2, pair.default_air_params(precision=precision, max_coarse=1000,
+                                                                      coarse_sweeps=sweeps))
+        x = h.vcycle(torch.as_tensor(np.tile(b, 2), device="cuda"), torch.zeros(2 * n, dtype=torch.float64, device="cuda"))
+        x = x.cpu().numpy()
+        assert np.array_equal(x[:n], x[n:])
+        assert np.linalg.norm(x[:n] - want) <= tol * max(np.linalg.norm(want), 1e-300)
