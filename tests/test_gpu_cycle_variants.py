@@ -39,7 +39,7 @@ def test_batch_size_does_not_change_the_flux(pair, mesh, n, precision, inner_tol
 
 # the coarsest sweeps as a dense product against plain sweeps: segments of one row, of
 # a row block and its neighbours, the largest, and one past it (which keeps the sweeps); the
-# two differ by the rounding of a few dozen additions
+# two differ by at most about n eps ||B|| / ||x|| sqrt(n) (n = 128: 3e-13, in FP32 1e-4)
 @pytest.mark.parametrize("n", [1, 3, 31, 32, 33, 97, 128, 129])
 @pytest.mark.parametrize("sweeps", [0, 1, 7])
 def test_coarsest_product_equals_sweeps(pair, n, sweeps):
@@ -54,7 +54,7 @@ def test_coarsest_product_equals_sweeps(pair, n, sweeps):
     want = np.zeros(n)
     for _ in range(sweeps):
         want = want + (b - A @ want) / np.diag(A)
-    for precision, tol in ((0, 1e-13), (1, 2e-6)):
+    for precision, tol in ((0, 1e-12), (1, 1e-4)):
         dev = [torch.as_tensor(a, device="cuda") for a in (rp, col, val)]
         h = pair.Hierarchy([tuple(dev)] * 2, pair.default_air_params(precision=precision, max_coarse=1000,
                                                                       coarse_sweeps=sweeps))
