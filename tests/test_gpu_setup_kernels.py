@@ -82,3 +82,15 @@ def test_lair_pattern_windows(pair):
         ci[s:e] = c
         va[s:e] = np.where(c == i, 1.0, g.uniform(0.5, 1.0, k + 1) / (4 * k))
     _check(pair, rp, ci, va, distance=2, theta=0.5, eps_R=0.001, max_levels=2)
+
+
+@pytest.mark.parametrize("entries,n", [
+    (6, 127), (14, 300),      # staged rows, a block's remainder
+    (30, 257), (40, 400),     # at and past the longest staged row
+    (120, 700), (140, 700),   # at and past the first hash table
+    (900, 1500),              # the second
+    (3000, 1500),             # longer rows, in their own slots
+])
+def test_galerkin_row_classes(pair, entries, n):
+    rp, ci, va = _matrix(n, lambda i: entries if i % 5 else 3, 40 + entries)
+    _check(pair, rp, ci, va, distance=1, theta=0.99, eps_R=0.97, max_levels=2, max_coarse=10)
