@@ -441,10 +441,9 @@ __global__ void __launch_bounds__(256) k_lair_pattern2_big(const int *big, const
     }
 }
 
-// lAIR systems binned by size: a thread per system up to 8 unknowns (bins of 4, 6
-// and 8, whose shared workspaces keep more systems in flight per SM the smaller
-// they are), 8 lanes per system up to 16, then a warp per system with a
-// shared-memory workspace sized to the bin, global workspaces beyond 64
+// lAIR systems binned by size, 4, 8, 16 or 32 lanes to a system of up to 8, 16, 32 or 64
+// unknowns, with shared workspaces sized to the bin (the smaller they are, the more
+// systems are in flight per SM); global workspaces beyond 64
 constexpr int LAIR_CLASSES = 10;
 constexpr int LAIR_BIG = LAIR_CLASSES - 1;
 __device__ __forceinline__ int lair_class(int np) {
@@ -554,138 +553,6 @@ __device__ __forceinline__ double times_recip(double y, double r) {
     if ((rb & 0x7fffffffffffffffLL) == 0x3ff0000000000000LL)
         return __longlong_as_double(__double_as_longlong(y) ^ (rb & (long long)0x8000000000000000ULL));
     return y * r;
-}
-
-// Thread per C row of the worklist for systems of size <= NM: every lane of a
-// warp works on its own system, so each FP64 instruction carries 32 useful
-// operations.  Workspaces live in shared memory interleaved by thread
-// (element e of thread t at [e * T + t]), which keeps accesses conflict-free.
-template <int NM>
-__global__ void __launch_bounds__(64) k_lair_solve_thread(int nwork, const int *worklist, const int *cpts,
-                                                          const int *rowptr, const int *col, const double *val,
-                                                          const int *candptr, const int *cand, const int *npat,
-                                                          const int *zrowptr, int *zcol, double *zval, int *keep,
-                                                          int *nsing_dir, const int *rowdir, double phi_R) {
-    constexpr int T = 64;
-    extern __shared__ double sm3[];
-    const int t = threadIdx.x;
-    double *Ms = sm3;                   // NM*NM
-    double *ys = sm3 + NM * NM * T;     // NM
-    double *rs = ys + NM * T;           // NM
-    int *ps = (int *)(rs + NM * T);     // NM pattern, NM pivots
-#define MM(e) Ms[(e) * T + t]
-#define YY(e) ys[(e) * T + t]
-#define RR(e) rs[(e) * T + t]
-#define PAT(e) ps[(e) * T + t]
-#define PIV(e) ps[(NM + (e)) * T + t]
-    int w = blockIdx.x * T + t;
-    if (w >= nwork) return;
-    int ic = worklist[w];
-    int i = cpts[ic];
-    int np = npat[ic];
-    if (np > NM) { keep[ic] = 0; return; }   // excluded by the size bins
-    const int *cp = cand + candptr[ic];
-    for (int e = 0; e < np; ++e) { PAT(e) = cp[e]; YY(e) = -0.0; }
-    for (int e = 0; e < np * np; ++e) MM(e) = 0.0;
-    for (int c = 0; c < np; ++c) {
-        const int j = PAT(c), p1 = rowptr[j + 1];
-        for (int p = rowptr[j]; p < p1; p += 4) {   // four entries' loads before their lookups
-            int kk[4];
-            double vv[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                kk[u] = p + u < p1 ? col[p + u] : -1;
-                vv[u] = p + u < p1 ? val[p + u] : 0.0;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int k = kk[u];
-                if (k < 0) continue;
-                int lo = 0, hi = np - 1, r = -1;
-                while (lo <= hi) {
-                    int m = (lo + hi) >> 1;
-                    int v = PAT(m);
-                    if (v == k) { r = m; break; }
-                    if (v < k) lo = m + 1; else hi = m - 1;
-                }
-                if (r >= 0) MM(r * np + c) = vv[u];
-            }
-        }
-    }
-    for (int p = rowptr[i]; p < rowptr[i + 1]; ++p) {
-        int k = col[p], lo = 0, hi = np - 1, r = -1;
-        while (lo <= hi) {
-            int m = (lo + hi) >> 1;
-            int v = PAT(m);
-            if (v == k) { r = m; break; }
-            if (v < k) lo = m + 1; else hi = m - 1;
-        }
-        if (r >= 0) YY(r) = -val[p];
-    }
-    long long mxb = 0;
-    for (int e = 0; e < np * np; ++e) mxb = max(mxb, absbits(MM(e)));
-    long long tinyb = absbits(1e-14 * __longlong_as_double(mxb));
-    bool singular = false;
-    for (int k = 0; k < np; ++k) {
-        int p = k;
-        long long pv = absbits(MM(k * np + k));
-        for (int r = k + 1; r < np; ++r) {
-            long long v = absbits(MM(r * np + k));
-            if (v > pv) { pv = v; p = r; }
-        }
-        PIV(k) = p;
-        if (!(pv > tinyb)) { singular = true; break; }
-        if (p != k)
-            for (int c = 0; c < np; ++c) { double tt = MM(k * np + c); MM(k * np + c) = MM(p * np + c); MM(p * np + c) = tt; }
-        double rd = pivot_recip(MM(k * np + k));
-        RR(k) = rd;
-        for (int r = k + 1; r < np; ++r) {
-            const double a = MM(r * np + k);
-            if (is_zero_bits(a)) {   // adds exact zeros: skipped, as in the reference LU
-                MM(r * np + k) = zero_times(a, rd);
-                continue;
-            }
-            const double l = a * rd;
-            MM(r * np + k) = l;
-            if (is_zero_bits(l)) continue;   // (an underflowed multiplier likewise)
-            for (int c = k + 1; c < np; ++c) MM(r * np + c) = fma(-l, MM(k * np + c), MM(r * np + c));
-        }
-    }
-    int kept = 0;
-    if (singular) {
-        atomicAdd(&nsing_dir[rowdir[i]], 1);
-    } else if (np > 0) {
-        for (int k = 0; k < np; ++k) {
-            int p = PIV(k);
-            if (p != k) { double tt = YY(k); YY(k) = YY(p); YY(p) = tt; }
-        }
-        for (int k = 0; k < np; ++k) {
-            double yk = YY(k);
-            for (int r = k + 1; r < np; ++r) YY(r) = fma(-MM(r * np + k), yk, YY(r));
-        }
-        for (int k = np - 1; k >= 0; --k) {
-            double yk = times_recip(YY(k), RR(k));
-            YY(k) = yk;
-            for (int r = 0; r < k; ++r) YY(r) = fma(-MM(r * np + k), yk, YY(r));
-        }
-        long long zmb = 0;
-        for (int e = 0; e < np; ++e) zmb = max(zmb, absbits(YY(e)));
-        double thr = phi_R * __longlong_as_double(zmb);
-        int base = zrowptr[ic];
-        for (int e = 0; e < np; ++e) {
-            double z = YY(e);
-            if (phi_R > 0.0 && fabs(z) < thr) continue;
-            zcol[base + kept] = PAT(e);
-            zval[base + kept] = z;
-            ++kept;
-        }
-    }
-    keep[ic] = kept;
-#undef MM
-#undef YY
-#undef RR
-#undef PAT
-#undef PIV
 }
 
 // G lanes per C row of the worklist (32/G systems per warp).  Shared-memory
@@ -918,6 +785,291 @@ __global__ void k_lair_solve(int nwork, const int *worklist, const int *cpts, co
                 zval[base + off] = y[t];
             }
             kept += __popc(msk);
+        }
+        if (has && g == 0) {
+            if (singular) atomicAdd(&nsing_dir[rowdir[i]], 1);
+            keep[ic] = solve ? kept : 0;
+        }
+        __syncwarp();
+    }
+}
+
+// Systems of up to 64 unknowns on column masks.  G lanes take a system (32 / G systems a
+// warp), lane g the columns g and g + G and the same entries of y; cm holds, per column,
+// the rows that may be nonzero.  The local matrices are A_FF restricted to a neighbourhood
+// of an upwind operator: a few entries per row, almost nothing below the diagonal, so with
+// the masks a pivot step whose column has no row below costs a shuffle of its mask instead
+// of a scan of the column, and elimination, fill-in and both substitutions touch stored
+// entries only.  Entries outside the masks are never read (the workspace is not cleared)
+// and stand for +0.0; forward substitution runs with the elimination, so L is not kept.
+//
+// The results are those of the dense elimination bit for bit.  What a dense pass does with
+// a zero is kept: a zero multiplier takes the sign of the pivot, and y - 0 * y_k changes
+// only the sign of a zero y (-0.0 becomes +0.0 when the product is +0.0), unless y_k is
+// not finite.
+//
+// Measured against the dense kernels (a thread a system up to 8 unknowns, 8 to 32 lanes on
+// cleared workspaces beyond): 64^3 S8 1311 -> 1232 ms (79 of 210 ms of local solves; the
+// three smallest bins alone 41 ms), an 18^3 x 6 tet matrix 29.6 -> 25.6 ms.
+// What bounds it: each FP64 warp instruction holds the SM's FP64 pipe for 16 cycles
+// whatever its active lanes, and the dense passes issued one per column, row and step; the
+// workspaces (odd row stride: columns are read without bank conflicts) set the resident
+// warps.
+__device__ __forceinline__ double sub_zero_product(double y, bool neg_zero_factor, double yk) {
+    // y - z * yk for a zero z (negative: neg_zero_factor)
+    const long long kb = __double_as_longlong(yk);
+    if ((kb & 0x7ff0000000000000LL) == 0x7ff0000000000000LL) return fma(neg_zero_factor ? 0.0 : -0.0, yk, y);
+    const bool plus = neg_zero_factor != (kb < 0);   // the product -z * yk is +0.0
+    return (plus && __double_as_longlong(y) == (long long)0x8000000000000000ULL) ? 0.0 : y;
+}
+
+template <int G>
+__global__ void k_lair_solve_mask(int nwork, const int *worklist, const int *cpts, const int *rowptr, const int *col,
+                                  const double *val, const int *candptr, const int *cand, const int *npat,
+                                  const int *zrowptr, int *zcol, double *zval, int *keep, int *nsing_dir,
+                                  const int *rowdir, double phi_R, int nmax) {
+    typedef unsigned long long u64;
+    constexpr int PN = 2 * G;     // pattern slots: a power of two >= nmax
+    constexpr int SPW = 32 / G;   // systems per warp
+    extern __shared__ double smem[];
+    const unsigned FULL = 0xffffffffu;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+    const int g = lane % G, q = lane / G, q0 = q * G;
+    const unsigned gmask = G == 32 ? FULL : ((1u << (G & 31)) - 1u);   // (shifted down to the group)
+    const int ld = nmax | 1;
+    double *M = smem + ((size_t)warp * SPW + q) * ((size_t)nmax * ld + nmax + G);
+    double *ys = M + (size_t)nmax * ld;
+    int *pat = (int *)(ys + nmax);
+    auto find = [&](int k) {   // position of column k in the pattern, or -1
+        int pos = 0;
+#pragma unroll
+        for (int h = G; h > 0; h >>= 1)
+            if (pat[pos + h - 1] < k) pos += h;
+        return pat[pos] == k ? pos : -1;
+    };
+    auto bcast_mask = [&](const u64 (&cm)[2], int k) {
+        return __shfl_sync(FULL, k < G ? cm[0] : cm[1], q0 + (k & (G - 1)));
+    };
+    auto bcast = [&](const double (&v)[2], int k) {
+        return __shfl_sync(FULL, k < G ? v[0] : v[1], q0 + (k & (G - 1)));
+    };
+    for (int wb = (blockIdx.x * wpb + warp) * SPW; wb < nwork; wb += gridDim.x * wpb * SPW) {
+        const int w = wb + q;
+        const bool has = w < nwork;
+        const int ic = has ? worklist[w] : 0;
+        const int i = has ? cpts[ic] : 0;
+        const int np = has ? npat[ic] : 0;
+        const int *cp = has ? cand + candptr[ic] : nullptr;
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const int c = g + G * t;
+            pat[c] = c < np ? cp[c] : 0x7fffffff;
+            if (c < np) ys[c] = -0.0;
+        }
+        __syncwarp();
+        // column c of the system is row pat[c] of A: four entries' loads before their lookups
+        u64 cm[2] = {0, 0};
+        long long mxb = 0;
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const int c = g + G * t;
+            if (c >= np) continue;
+            const int j = pat[c], p1 = rowptr[j + 1];
+            for (int p = rowptr[j]; p < p1; p += 4) {
+                int cc[4], r[4];
+                double vv[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    cc[u] = p + u < p1 ? col[p + u] : -1;
+                    vv[u] = p + u < p1 ? val[p + u] : 0.0;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) r[u] = find(cc[u]);
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (r[u] >= 0) {
+                        M[r[u] * ld + c] = vv[u];
+                        cm[t] |= 1ULL << r[u];
+                        mxb = max(mxb, absbits(vv[u]));
+                    }
+            }
+        }
+        if (has)
+            for (int p = rowptr[i] + g; p < rowptr[i + 1]; p += G) {
+                const int r = find(col[p]);
+                if (r >= 0) ys[r] = -val[p];
+            }
+        __syncwarp();
+        double y[2];
+#pragma unroll
+        for (int t = 0; t < 2; ++t) y[t] = g + G * t < np ? ys[g + G * t] : 0.0;
+        int kmax = np;
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) mxb = max(mxb, __shfl_xor_sync(FULL, mxb, o, G));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) kmax = max(kmax, __shfl_xor_sync(FULL, kmax, o));
+        const long long tinyb = absbits(1e-14 * __longlong_as_double(mxb));
+        bool singular = false;
+        for (int k = 0; k < kmax; ++k) {
+            bool act = k < np && !singular;
+            u64 mk = bcast_mask(cm, k);
+            if (!act) mk = 0;
+            double pk = (mk >> k) & 1 ? M[k * ld + k] : 0.0;
+            const u64 above = (2ULL << k) - 1ULL;   // rows 0..k
+            const bool need = (mk & ~above) != 0;
+            long long bv = absbits(pk);
+            int br = k;
+            const bool step = __any_sync(FULL, need);
+            double a[2] = {0.0, 0.0};
+            if (step) {   // pivot: the first largest magnitude of rows k.. (unstored rows are zero)
+                if (need) {
+                    bv = -1;
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        const int r = g + G * t;
+                        if (r < k || r >= np) continue;
+                        const long long v = (mk >> r) & 1 ? absbits(M[r * ld + k]) : 0;
+                        if (v > bv) { bv = v; br = r; }
+                    }
+                }
+#pragma unroll
+                for (int o = G / 2; o > 0; o >>= 1) {
+                    const long long ov = __shfl_xor_sync(FULL, bv, o, G);
+                    const int orr = __shfl_xor_sync(FULL, br, o, G);
+                    if (ov > bv || (ov == bv && orr < br)) { bv = ov; br = orr; }
+                }
+            }
+            if (act && !(bv > tinyb)) { singular = true; act = false; }
+            const bool elim = act && need;
+            if (step) {
+                const bool swp = elim && br != k;
+                if (__any_sync(FULL, swp)) {
+                    const double yk0 = bcast(y, k);
+                    const double b0 = __shfl_sync(FULL, y[0], q0 + (br & (G - 1)));
+                    const double b1 = __shfl_sync(FULL, y[1], q0 + (br & (G - 1)));
+                    if (swp) {
+#pragma unroll
+                        for (int t = 0; t < 2; ++t) {
+                            const int c = g + G * t;
+                            if (c < np) {
+                                const double tv = M[k * ld + c];
+                                M[k * ld + c] = M[br * ld + c];
+                                M[br * ld + c] = tv;
+                            }
+                            if (c == k) y[t] = br < G ? b0 : b1;
+                            else if (c == br) y[t] = yk0;
+                            const u64 x = ((cm[t] >> k) ^ (cm[t] >> br)) & 1ULL;
+                            cm[t] ^= (x << k) | (x << br);
+                        }
+                        const u64 x = ((mk >> k) ^ (mk >> br)) & 1ULL;
+                        mk ^= (x << k) | (x << br);
+                    }
+                    __syncwarp();
+                    if (swp) pk = M[k * ld + k];
+                }
+            }
+            const double yk = bcast(y, k);
+            const bool negp = __double_as_longlong(pk) < 0;   // the sign of a zero multiplier
+            if (!step) {
+                if (act)
+#pragma unroll
+                    for (int t = 0; t < 2; ++t)
+                        if (g + G * t > k) y[t] = sub_zero_product(y[t], negp, yk);
+                continue;
+            }
+            // the pivot's reciprocal: one lane of the group divides
+            double rd = 0.0;
+            if (elim && g == 0) rd = pivot_recip(pk);
+            rd = __shfl_sync(FULL, rd, q0);
+            u64 Lm = 0;   // rows whose multiplier is not zero
+            double l[2];
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                const int r = g + G * t;
+                const bool inb = elim && r > k && ((mk >> r) & 1);
+                a[t] = inb ? M[r * ld + k] : 0.0;
+                const bool nz = inb && !is_zero_bits(a[t]);
+                l[t] = nz ? a[t] * rd : 0.0;
+                const bool upd = nz && !is_zero_bits(l[t]);
+                if (act && r > k) {
+                    if (upd) y[t] = fma(-l[t], yk, y[t]);
+                    else {
+                        // zero multiplier: zero entry times the reciprocal, or an underflow
+                        const bool neg = nz ? __double_as_longlong(l[t]) < 0 : (__double_as_longlong(a[t]) < 0) != negp;
+                        y[t] = sub_zero_product(y[t], neg, yk);
+                    }
+                }
+                const unsigned b = (__ballot_sync(FULL, upd) >> q0) & gmask;
+                Lm |= (u64)b << (G * t);
+            }
+            u64 rem = Lm;
+            while (__any_sync(FULL, rem != 0)) {
+                const int r = rem ? __ffsll((long long)rem) - 1 : 0;
+                const double l0 = __shfl_sync(FULL, l[0], q0 + (r & (G - 1)));
+                const double l1 = __shfl_sync(FULL, l[1], q0 + (r & (G - 1)));
+                if (rem) {
+                    const double lr = r < G ? l0 : l1;
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        const int c = g + G * t;
+                        const bool bk = (cm[t] >> k) & 1, brr = (cm[t] >> r) & 1;
+                        if (c > k && c < np && (bk || brr)) {
+                            const double mv = brr ? M[r * ld + c] : 0.0, bkv = bk ? M[k * ld + c] : 0.0;
+                            M[r * ld + c] = fma(-lr, bkv, mv);
+                        }
+                    }
+                }
+                rem &= rem - 1;
+            }
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+                if (g + G * t > k && ((cm[t] >> k) & 1)) cm[t] |= Lm;
+            __syncwarp();
+        }
+        const bool solve = has && !singular && np > 0;
+        double rv[2];
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const int c = g + G * t;
+            rv[t] = solve && c < np ? pivot_recip(M[c * ld + c]) : 1.0;
+        }
+        for (int k = kmax - 1; k >= 0; --k) {
+            const bool act = solve && k < np;
+            const u64 mk = bcast_mask(cm, k);
+            if (act && g == (k & (G - 1))) {
+                if (k < G) y[0] = times_recip(y[0], rv[0]);
+                else y[1] = times_recip(y[1], rv[1]);
+            }
+            const double yk = bcast(y, k);
+            if (act)
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    const int r = g + G * t;
+                    if (r >= k) continue;
+                    if ((mk >> r) & 1) y[t] = fma(-M[r * ld + k], yk, y[t]);
+                    else y[t] = sub_zero_product(y[t], false, yk);
+                }
+        }
+        long long zmb = 0;
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+            if (solve && g + G * t < np) zmb = max(zmb, absbits(y[t]));
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) zmb = max(zmb, __shfl_xor_sync(FULL, zmb, o, G));
+        const double thr = phi_R * __longlong_as_double(zmb);
+        const int base = has ? zrowptr[ic] : 0;
+        int kept = 0;
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const int c = g + G * t;
+            const bool k_ = solve && c < np && !(phi_R > 0.0 && fabs(y[t]) < thr);
+            const unsigned b = (__ballot_sync(FULL, k_) >> q0) & gmask;
+            if (k_) {
+                const int off = kept + __popc(b & ((1u << g) - 1u));
+                zcol[base + off] = pat[c];
+                zval[base + off] = y[t];
+            }
+            kept += __popc(b);
         }
         if (has && g == 0) {
             if (singular) atomicAdd(&nsing_dir[rowdir[i]], 1);
@@ -1859,17 +2011,6 @@ void build_hierarchy(Hier &h) {
             int *list = dmalloc<int>(nc, s);
             partition_by_class(ccls, nc, LAIR_CLASSES, list, hstart, hc, s);
             dfree(ccls, s);
-            // n <= 8: a thread per system; 9..24 unknowns: 32 / G systems per warp (G = 8
-            // lanes each up to 16 unknowns, 16 lanes up to 24); larger: a warp per system
-            auto thread_bin = [&](int c, auto kern, int nm) {
-                if (!hc[c]) return;
-                size_t sm = (size_t)64 * (nm * nm + 3 * nm) * sizeof(double);
-                if (sm > 48 * 1024) allow_max_dyn_smem(kern);
-                kern<<<blocks_for(hc[c], 64), 64, sm, s>>>(hc[c], list + hstart[c], L.cpts, L.rowptr, L.col, L.val,
-                                                           candptr, cand, npat, zr, zc, zv, keep, dsing, L.rowdir,
-                                                           prm.phi_R);
-                PR_LAUNCH();
-            };
             const int cls_n[LAIR_CLASSES] = {4, 6, 8, 12, 16, 24, 32, 48, 64, 0};
             int smem_optin = 0;
             {
@@ -1877,31 +2018,27 @@ void build_hierarchy(Hier &h) {
                 PR_CUDA(cudaGetDevice(&dev));
                 PR_CUDA(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
             }
-            auto warp_bin = [&](int c, auto kern, int G) {
+            auto mask_bin = [&](int c, auto kern, int G) {
                 if (!hc[c]) return;
                 const int nm = cls_n[c], spw = 32 / G;
-                size_t per = ((size_t)nm * nm + 4 * nm) * sizeof(double) * spw;   // per warp
-                // as many warps per block as the shared memory of one block holds (the
-                // solves are latency- and FP64-bound, so resident warps decide)
-                int wpb = (int)std::max<size_t>(1, std::min<size_t>(32, (size_t)smem_optin / per));
-                cudaFuncAttributes fa;   // and no more threads than its registers allow
-                PR_CUDA(cudaFuncGetAttributes(&fa, kern));
-                wpb = std::max(1, std::min(wpb, fa.maxThreadsPerBlock / 32));
-                size_t sm = per * wpb;
-                unsigned grid = std::min<unsigned>(blocks_for(hc[c], wpb * spw), 152u * 64u);
+                const size_t per = ((size_t)nm * (nm | 1) + nm + G) * sizeof(double) * spw;   // per warp
+                // blocks of up to four warps: many small blocks fill the SM's shared memory
+                // (and so its resident warps) evenly
+                const int wpb = (int)std::max<size_t>(1, std::min<size_t>(4, (size_t)smem_optin / per));
+                const size_t sm = per * wpb;
+                const unsigned grid = std::min<unsigned>(blocks_for(hc[c], wpb * spw), 152u * 256u);
                 if (sm > 48 * 1024) allow_max_dyn_smem(kern);
                 kern<<<grid, 32 * wpb, sm, s>>>(hc[c], list + hstart[c], L.cpts, L.rowptr, L.col, L.val, candptr,
-                                                cand, npat, zr, zc, zv, keep, dsing, L.rowdir, prm.phi_R, nm, nullptr,
-                                                nullptr);
+                                                cand, npat, zr, zc, zv, keep, dsing, L.rowdir, prm.phi_R, nm);
                 PR_LAUNCH();
             };
-            thread_bin(0, k_lair_solve_thread<4>, 4);
-            thread_bin(1, k_lair_solve_thread<6>, 6);
-            thread_bin(2, k_lair_solve_thread<8>, 8);
-            warp_bin(3, k_lair_solve<8>, 8);
-            warp_bin(4, k_lair_solve<8>, 8);
-            warp_bin(5, k_lair_solve<16>, 16);
-            for (int c = 6; c < LAIR_BIG; ++c) warp_bin(c, k_lair_solve<32>, 32);
+            for (int c = 0; c <= 2; ++c) mask_bin(c, k_lair_solve_mask<4>, 4);
+            mask_bin(3, k_lair_solve_mask<8>, 8);
+            mask_bin(4, k_lair_solve_mask<8>, 8);
+            mask_bin(5, k_lair_solve_mask<16>, 16);
+            mask_bin(6, k_lair_solve_mask<16>, 16);
+            mask_bin(7, k_lair_solve_mask<32>, 32);
+            mask_bin(8, k_lair_solve_mask<32>, 32);
             int nbig = hc[LAIR_BIG];
             if (nbig > 0) {
                 long long *goff = dmalloc<long long>(nbig + 1, s);

@@ -94,3 +94,32 @@ def test_lair_pattern_windows(pair):
 def test_galerkin_row_classes(pair, entries, n):
     rp, ci, va = _matrix(n, lambda i: entries if i % 5 else 3, 40 + entries)
     _check(pair, rp, ci, va, distance=1, theta=0.99, eps_R=0.97, max_levels=2, max_coarse=10)
+
+
+def _coupled(n, entries, seed):
+    """Rows of `entries` neighbours in a band, small and zero diagonals, stored zeros of both
+    signs: local systems that exchange rows, fill in, and are sometimes singular."""
+    g = np.random.default_rng(seed)
+    rp, ci, va = [0], [], []
+    for i in range(n):
+        lo, hi = max(0, i - entries), min(n, i + entries + 1)
+        c = np.unique(np.append(g.choice(np.arange(lo, hi), min(entries, hi - lo), replace=False), i))
+        v = g.uniform(-1.0, 1.0, c.size)
+        z = g.random(c.size)
+        v[z < 0.15] = 0.0
+        v[z < 0.07] = -0.0
+        v[c == i] = g.choice([1.0, 0.3, -0.2, 0.0 if i % 7 == 0 else 0.5])
+        rp.append(rp[-1] + c.size)
+        ci.append(c)
+        va.append(v)
+    return np.array(rp, np.int32), np.concatenate(ci).astype(np.int32), np.concatenate(va)
+
+
+@pytest.mark.parametrize("phi_R", [0.0, 0.1])
+@pytest.mark.parametrize("entries,distance", [(3, 1), (6, 1), (9, 1), (14, 1), (22, 1), (34, 1), (55, 1), (80, 1),
+                                              (3, 2), (5, 2), (8, 2)])
+def test_lair_solver_bins(pair, entries, distance, phi_R):
+    """Local systems of every size class (up to 4, 6, 8, 12, 16, 24, 32, 48, 64 and more
+    unknowns) that need pivoting."""
+    rp, ci, va = _coupled(500, entries, 60 + entries)
+    _check(pair, rp, ci, va, distance=distance, theta=0.6, phi_R=phi_R, max_levels=2, max_coarse=10)
