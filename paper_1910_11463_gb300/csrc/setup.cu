@@ -1367,54 +1367,44 @@ __global__ void k_rap(int nrows_work, const int *worklist, const int *cpts, cons
             __syncwarp();
             k_c = k_n; r_c = r_n; a_c = a_n; l_c = l_n; c_c = c_n; v_c = v_n;
         }
-        // compact to the scratch output (unsorted), then rank-sort back into the table
-        int base = has ? uptr[ic] : 0;
-        int m = 0;
-        int capmax = cap;
-        for (int o = 16; o > 0; o >>= 1) capmax = max(capmax, __shfl_xor_sync(FULL, capmax, o));
-        for (int s0 = 0; s0 < capmax; s0 += G) {
-            int sl = s0 + g;
-            bool occ = sl < cap && keys[sl] >= 0;
-            unsigned msk = __ballot_sync(FULL, occ) & gmask;
-            if (occ) {
-                int off = m + __popc(msk & ((1u << lane) - 1u));
-                ucol[base + off] = keys[sl];
-                uval[base + off] = vals[sl];
-            }
-            m += __popc(msk);
-        }
-        __syncwarp();
-        for (int e = g; e < m; e += G) {
-            int ce = ucol[base + e];
-            int rank = 0;
-            for (int f = 0; f < m; ++f) rank += ucol[base + f] < ce;
-            keys[rank] = ce;
-            vals[rank] = uval[base + e];
-        }
-        __syncwarp();
-        int mmax = m;
-        for (int o = 16; o > 0; o >>= 1) mmax = max(mmax, __shfl_xor_sync(FULL, mmax, o));
+        const int base = has ? uptr[ic] : 0;
+        // The phi_A filter (threshold from the table), then the kept entries are packed in
+        // the table itself and each is written at its column's rank among them, once.
+        // (Ranking from an unsorted list in the output arrays read every column through L2
+        // right after it was written, and the filter took another pass.)
         double thr = 0.0;
         if (filt) {
             long long mxb = 0;
-            for (int e = g; e < m; e += G)
-                if (keys[e] != ic) mxb = max(mxb, absbits(vals[e]));
+            for (int sl = g; sl < cap; sl += G)
+                if (keys[sl] >= 0 && keys[sl] != ic) mxb = max(mxb, absbits(vals[sl]));
             for (int o = G / 2; o > 0; o >>= 1) mxb = max(mxb, __shfl_xor_sync(FULL, mxb, o, G));
             thr = phiA * __longlong_as_double(mxb);
         }
-        int kept = 0;
-        for (int e0 = 0; e0 < mmax; e0 += G) {
-            int e = e0 + g;
-            bool k_ = e < m && !(filt && keys[e] != ic && fabs(vals[e]) < thr);
-            unsigned msk = __ballot_sync(FULL, k_) & gmask;
+        int m = 0;
+        int capmax = cap;
+        for (int o = 16; o > 0; o >>= 1) capmax = max(capmax, __shfl_xor_sync(FULL, capmax, o));
+        for (int s0 = 0; s0 < capmax; s0 += G) {   // kept entries move to the table's front
+            const int sl = s0 + g;
+            const int key = sl < cap ? keys[sl] : -1;
+            const double v = sl < cap ? vals[sl] : 0.0;
+            const bool k_ = key >= 0 && !(filt && key != ic && fabs(v) < thr);
+            const unsigned msk = __ballot_sync(FULL, k_) & gmask;   // (every slot of the pass is read)
             if (k_) {
-                int off = kept + __popc(msk & ((1u << lane) - 1u));
-                ucol[base + off] = keys[e];
-                uval[base + off] = vals[e];
+                const int off = m + __popc(msk & ((1u << lane) - 1u));
+                keys[off] = key;
+                vals[off] = v;
             }
-            kept += __popc(msk);
+            m += __popc(msk);
+            __syncwarp();
         }
-        if (has && g == 0) cnt[ic] = kept;
+        for (int e = g; e < m; e += G) {
+            const int ce = keys[e];
+            int rank = 0;
+            for (int f = 0; f < m; ++f) rank += keys[f] < ce;
+            ucol[base + rank] = ce;
+            uval[base + rank] = vals[e];
+        }
+        if (has && g == 0) cnt[ic] = m;
         __syncwarp();
     }
 }
