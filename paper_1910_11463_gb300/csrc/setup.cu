@@ -443,12 +443,12 @@ __global__ void __launch_bounds__(256) k_lair_pattern2_big(const int *big, const
 
 // lAIR systems binned by size, 4, 8, 16 or 32 lanes to a system of up to 8, 16, 32 or 64
 // unknowns, with shared workspaces sized to the bin (the smaller they are, the more
-// systems are in flight per SM); global workspaces beyond 64
-constexpr int LAIR_CLASSES = 10;
+// systems are in flight per SM); global workspaces beyond 64, and a dense kernel past 256
+constexpr int LAIR_CLASSES = 12;
 constexpr int LAIR_BIG = LAIR_CLASSES - 1;
 __device__ __forceinline__ int lair_class(int np) {
     return np <= 4 ? 0 : np <= 6 ? 1 : np <= 8 ? 2 : np <= 12 ? 3 : np <= 16 ? 4 : np <= 24 ? 5 : np <= 32 ? 6
-         : np <= 48 ? 7 : np <= 64 ? 8 : 9;
+         : np <= 48 ? 7 : np <= 64 ? 8 : np <= 128 ? 9 : np <= 256 ? 10 : 11;
 }
 
 
@@ -555,15 +555,13 @@ __device__ __forceinline__ double times_recip(double y, double r) {
     return y * r;
 }
 
-// G lanes per C row of the worklist (32/G systems per warp).  Shared-memory
-// mode (gbuf == null): systems of size <= nmax, workspace nmax^2 + 2 nmax
-// doubles per group.  Global mode: workspace at gbuf + goff[w].
-template <int G>
-__global__ void k_lair_solve(int nwork, const int *worklist, const int *cpts, const int *rowptr, const int *col,
+// Systems past the mask kernels' largest: a warp per system, dense, workspace at
+// gbuf + goff[w].
+__global__ void k_lair_solve_dense(int nwork, const int *worklist, const int *cpts, const int *rowptr, const int *col,
                              const double *val, const int *candptr, const int *cand, const int *npat,
                              const int *zrowptr, int *zcol, double *zval, int *keep, int *nsing_dir,
-                             const int *rowdir, double phi_R, int nmax, const long long *goff, double *gbuf) {
-    extern __shared__ double smem[];
+                                   const int *rowdir, double phi_R, const long long *goff, double *gbuf) {
+    constexpr int G = 32;
     const unsigned FULL = 0xffffffffu;
     int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int g = lane % G, q = lane / G;
@@ -576,8 +574,7 @@ __global__ void k_lair_solve(int nwork, const int *worklist, const int *cpts, co
         int ic = has ? worklist[w] : 0;
         int i = has ? cpts[ic] : 0;
         int np = has ? npat[ic] : 0;
-        double *M = gbuf ? gbuf + (has ? goff[w] : 0)
-                         : smem + ((size_t)warp * SPW + q) * ((size_t)nmax * nmax + 4 * nmax);
+        double *M = gbuf + (has ? goff[w] : 0);
         double *y = M + (size_t)np * np;
         double *rv = y + np;                  // pivot reciprocals
         int *pat = (int *)(rv + np);
@@ -794,8 +791,8 @@ __global__ void k_lair_solve(int nwork, const int *worklist, const int *cpts, co
     }
 }
 
-// Systems of up to 64 unknowns on column masks.  G lanes take a system (32 / G systems a
-// warp), lane g the columns g and g + G and the same entries of y; cm holds, per column,
+// Systems of up to 256 unknowns on column masks.  G lanes take a system (32 / G systems a
+// warp), lane g the columns g, g + G, ... and the same entries of y; cm holds, per column,
 // the rows that may be nonzero.  The local matrices are A_FF restricted to a neighbourhood
 // of an upwind operator: a few entries per row, almost nothing below the diagonal, so with
 // the masks a pivot step whose column has no row below costs a shuffle of its mask instead
@@ -810,7 +807,8 @@ __global__ void k_lair_solve(int nwork, const int *worklist, const int *cpts, co
 //
 // Measured against the dense kernels (a thread a system up to 8 unknowns, 8 to 32 lanes on
 // cleared workspaces beyond): 64^3 S8 1311 -> 1232 ms (79 of 210 ms of local solves; the
-// three smallest bins alone 41 ms), an 18^3 x 6 tet matrix 29.6 -> 25.6 ms.
+// three smallest bins alone 41 ms), an 18^3 x 6 tet matrix 29.6 -> 25.6 ms; with the bins
+// past 64 unknowns and blocks small enough to fill an SM, 40^3 x 6 tets S4 537 -> 507 ms.
 // What bounds it: each FP64 warp instruction holds the SM's FP64 pipe for 16 cycles
 // whatever its active lanes, and the dense passes issued one per column, row and step; the
 // workspaces (odd row stride: columns are read without bank conflicts) set the resident
@@ -823,35 +821,91 @@ __device__ __forceinline__ double sub_zero_product(double y, bool neg_zero_facto
     return (plus && __double_as_longlong(y) == (long long)0x8000000000000000ULL) ? 0.0 : y;
 }
 
-template <int G>
+// W words of row bits; bit indices are per lane or uniform, word indices constants
+template <int W>
+struct RowMask {
+    unsigned long long w[W];
+    __device__ __forceinline__ bool has(int r) const {
+        if (W == 1) return (w[0] >> r) & 1ULL;
+        bool b = false;
+#pragma unroll
+        for (int k = 0; k < W; ++k)
+            if ((r >> 6) == k) b = (w[k] >> (r & 63)) & 1ULL;
+        return b;
+    }
+    __device__ __forceinline__ void flip(int r) {
+#pragma unroll
+        for (int k = 0; k < W; ++k)
+            if (W == 1 || (r >> 6) == k) w[k] ^= 1ULL << (r & 63);
+    }
+    // a row past r
+    __device__ __forceinline__ bool any_past(int r) const {
+        bool b = false;
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            const unsigned long long m = (r >> 6) == k ? w[k] & ~((2ULL << (r & 63)) - 1ULL) : (r >> 6) < k ? w[k] : 0ULL;
+            b |= m != 0;
+        }
+        return b;
+    }
+};
+
+// column k's mask, to every lane of its group (first lane q0)
+template <int G, int R, int W>
+__device__ __forceinline__ RowMask<W> mask_column(const RowMask<W> (&cm)[R], int k, int q0) {
+    RowMask<W> x;
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+        unsigned long long v = cm[0].w[j];
+#pragma unroll
+        for (int t = 1; t < R; ++t) {
+            const unsigned long long u = cm[t].w[j];
+            v = k / G == t ? u : v;
+        }
+        x.w[j] = __shfl_sync(0xffffffffu, v, q0 + (k & (G - 1)));
+    }
+    return x;
+}
+
+// G lanes, R columns a lane: systems of up to G R unknowns.  GLOBAL: the workspace is a
+// slot of gbuf per warp (systems of more than 64 unknowns; nothing is cleared and little is
+// touched, so the slots in use stay in L2), else shared memory.  M is column-major: a
+// column's rows are read by consecutive lanes.
+template <int G, int R, bool GLOBAL>
 __global__ void k_lair_solve_mask(int nwork, const int *worklist, const int *cpts, const int *rowptr, const int *col,
                                   const double *val, const int *candptr, const int *cand, const int *npat,
                                   const int *zrowptr, int *zcol, double *zval, int *keep, int *nsing_dir,
-                                  const int *rowdir, double phi_R, int nmax) {
+                                  const int *rowdir, double phi_R, int nmax, double *gbuf) {
     typedef unsigned long long u64;
-    constexpr int PN = 2 * G;     // pattern slots: a power of two >= nmax
+    constexpr int PN = R * G;     // pattern slots: a power of two >= nmax
     constexpr int SPW = 32 / G;   // systems per warp
+    constexpr int W = (PN + 63) / 64;
     extern __shared__ double smem[];
     const unsigned FULL = 0xffffffffu;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
     const int g = lane % G, q = lane / G, q0 = q * G;
     const unsigned gmask = G == 32 ? FULL : ((1u << (G & 31)) - 1u);   // (shifted down to the group)
     const int ld = nmax | 1;
-    double *M = smem + ((size_t)warp * SPW + q) * ((size_t)nmax * ld + nmax + G);
-    double *ys = M + (size_t)nmax * ld;
+    const size_t msz = (size_t)nmax * ld;
+    double *ws = smem + ((size_t)warp * SPW + q) * ((GLOBAL ? 0 : msz) + nmax + PN / 2);
+    double *M = GLOBAL ? gbuf + ((size_t)blockIdx.x * wpb + warp) * msz : ws;
+    double *ys = ws + (GLOBAL ? 0 : msz);
     int *pat = (int *)(ys + nmax);
     auto find = [&](int k) {   // position of column k in the pattern, or -1
         int pos = 0;
 #pragma unroll
-        for (int h = G; h > 0; h >>= 1)
+        for (int h = PN / 2; h > 0; h >>= 1)
             if (pat[pos + h - 1] < k) pos += h;
         return pat[pos] == k ? pos : -1;
     };
-    auto bcast_mask = [&](const u64 (&cm)[2], int k) {
-        return __shfl_sync(FULL, k < G ? cm[0] : cm[1], q0 + (k & (G - 1)));
-    };
-    auto bcast = [&](const double (&v)[2], int k) {
-        return __shfl_sync(FULL, k < G ? v[0] : v[1], q0 + (k & (G - 1)));
+    auto bcast = [&](const double (&v)[R], int k) {
+        double x = v[0];
+#pragma unroll
+        for (int t = 1; t < R; ++t) {
+            const double u = v[t];
+            x = k / G == t ? u : x;
+        }
+        return __shfl_sync(FULL, x, q0 + (k & (G - 1)));
     };
     for (int wb = (blockIdx.x * wpb + warp) * SPW; wb < nwork; wb += gridDim.x * wpb * SPW) {
         const int w = wb + q;
@@ -861,21 +915,22 @@ __global__ void k_lair_solve_mask(int nwork, const int *worklist, const int *cpt
         const int np = has ? npat[ic] : 0;
         const int *cp = has ? cand + candptr[ic] : nullptr;
 #pragma unroll
-        for (int t = 0; t < 2; ++t) {
+        for (int t = 0; t < R; ++t) {
             const int c = g + G * t;
             pat[c] = c < np ? cp[c] : 0x7fffffff;
             if (c < np) ys[c] = -0.0;
         }
         __syncwarp();
         // column c of the system is row pat[c] of A: four entries' loads before their lookups
-        u64 cm[2] = {0, 0};
+        RowMask<W> cm[R];
         long long mxb = 0;
 #pragma unroll
-        for (int t = 0; t < 2; ++t) {
-            const int c = g + G * t;
-            if (c >= np) continue;
-            const int j = pat[c], p1 = rowptr[j + 1];
-            for (int p = rowptr[j]; p < p1; p += 4) {
+        for (int t = 0; t < R; ++t) {
+            RowMask<W> x;
+#pragma unroll
+            for (int k = 0; k < W; ++k) x.w[k] = 0;
+            const int c = g + G * t, j = c < np ? pat[c] : 0, p1 = c < np ? rowptr[j + 1] : 0;
+            for (int p = c < np ? rowptr[j] : 0; p < p1; p += 4) {
                 int cc[4], r[4];
                 double vv[4];
 #pragma unroll
@@ -888,11 +943,12 @@ __global__ void k_lair_solve_mask(int nwork, const int *worklist, const int *cpt
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
                     if (r[u] >= 0) {
-                        M[r[u] * ld + c] = vv[u];
-                        cm[t] |= 1ULL << r[u];
+                        M[(size_t)c * ld + r[u]] = vv[u];
+                        x.flip(r[u]);   // (a row holds a column once)
                         mxb = max(mxb, absbits(vv[u]));
                     }
             }
+            cm[t] = x;
         }
         if (has)
             for (int p = rowptr[i] + g; p < rowptr[i + 1]; p += G) {
@@ -900,9 +956,9 @@ __global__ void k_lair_solve_mask(int nwork, const int *worklist, const int *cpt
                 if (r >= 0) ys[r] = -val[p];
             }
         __syncwarp();
-        double y[2];
+        double y[R];
 #pragma unroll
-        for (int t = 0; t < 2; ++t) y[t] = g + G * t < np ? ys[g + G * t] : 0.0;
+        for (int t = 0; t < R; ++t) y[t] = g + G * t < np ? ys[g + G * t] : 0.0;
         int kmax = np;
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) mxb = max(mxb, __shfl_xor_sync(FULL, mxb, o, G));
@@ -912,23 +968,21 @@ __global__ void k_lair_solve_mask(int nwork, const int *worklist, const int *cpt
         bool singular = false;
         for (int k = 0; k < kmax; ++k) {
             bool act = k < np && !singular;
-            u64 mk = bcast_mask(cm, k);
-            if (!act) mk = 0;
-            double pk = (mk >> k) & 1 ? M[k * ld + k] : 0.0;
-            const u64 above = (2ULL << k) - 1ULL;   // rows 0..k
-            const bool need = (mk & ~above) != 0;
+            RowMask<W> mk = mask_column<G, R, W>(cm, k, q0);
+            double *Mk = M + (size_t)k * ld;
+            double pk = act && mk.has(k) ? Mk[k] : 0.0;
+            const bool need = act && mk.any_past(k);
             long long bv = absbits(pk);
             int br = k;
             const bool step = __any_sync(FULL, need);
-            double a[2] = {0.0, 0.0};
             if (step) {   // pivot: the first largest magnitude of rows k.. (unstored rows are zero)
                 if (need) {
                     bv = -1;
 #pragma unroll
-                    for (int t = 0; t < 2; ++t) {
+                    for (int t = 0; t < R; ++t) {
                         const int r = g + G * t;
                         if (r < k || r >= np) continue;
-                        const long long v = (mk >> r) & 1 ? absbits(M[r * ld + k]) : 0;
+                        const long long v = mk.has(r) ? absbits(Mk[r]) : 0;
                         if (v > bv) { bv = v; br = r; }
                     }
                 }
@@ -945,27 +999,30 @@ __global__ void k_lair_solve_mask(int nwork, const int *worklist, const int *cpt
                 const bool swp = elim && br != k;
                 if (__any_sync(FULL, swp)) {
                     const double yk0 = bcast(y, k);
-                    const double b0 = __shfl_sync(FULL, y[0], q0 + (br & (G - 1)));
-                    const double b1 = __shfl_sync(FULL, y[1], q0 + (br & (G - 1)));
+                    double yb = 0.0;
+#pragma unroll
+                    for (int t = 0; t < R; ++t) {
+                        const double x = __shfl_sync(FULL, y[t], q0 + (br & (G - 1)));
+                        if (br / G == t) yb = x;
+                    }
                     if (swp) {
 #pragma unroll
-                        for (int t = 0; t < 2; ++t) {
+                        for (int t = 0; t < R; ++t) {
                             const int c = g + G * t;
                             if (c < np) {
-                                const double tv = M[k * ld + c];
-                                M[k * ld + c] = M[br * ld + c];
-                                M[br * ld + c] = tv;
+                                double *Mc = M + (size_t)c * ld;
+                                const double tv = Mc[k];
+                                Mc[k] = Mc[br];
+                                Mc[br] = tv;
                             }
-                            if (c == k) y[t] = br < G ? b0 : b1;
+                            if (c == k) y[t] = yb;
                             else if (c == br) y[t] = yk0;
-                            const u64 x = ((cm[t] >> k) ^ (cm[t] >> br)) & 1ULL;
-                            cm[t] ^= (x << k) | (x << br);
+                            if (cm[t].has(k) != cm[t].has(br)) { cm[t].flip(k); cm[t].flip(br); }
                         }
-                        const u64 x = ((mk >> k) ^ (mk >> br)) & 1ULL;
-                        mk ^= (x << k) | (x << br);
+                        if (mk.has(k) != mk.has(br)) { mk.flip(k); mk.flip(br); }
                     }
                     __syncwarp();
-                    if (swp) pk = M[k * ld + k];
+                    if (swp) pk = Mk[k];
                 }
             }
             const double yk = bcast(y, k);
@@ -973,7 +1030,7 @@ __global__ void k_lair_solve_mask(int nwork, const int *worklist, const int *cpt
             if (!step) {
                 if (act)
 #pragma unroll
-                    for (int t = 0; t < 2; ++t)
+                    for (int t = 0; t < R; ++t)
                         if (g + G * t > k) y[t] = sub_zero_product(y[t], negp, yk);
                 continue;
             }
@@ -981,78 +1038,90 @@ __global__ void k_lair_solve_mask(int nwork, const int *worklist, const int *cpt
             double rd = 0.0;
             if (elim && g == 0) rd = pivot_recip(pk);
             rd = __shfl_sync(FULL, rd, q0);
-            u64 Lm = 0;   // rows whose multiplier is not zero
-            double l[2];
+            RowMask<W> Lm;   // rows whose multiplier is not zero
 #pragma unroll
-            for (int t = 0; t < 2; ++t) {
+            for (int j = 0; j < W; ++j) Lm.w[j] = 0;
+            double l[R];
+#pragma unroll
+            for (int t = 0; t < R; ++t) {
                 const int r = g + G * t;
-                const bool inb = elim && r > k && ((mk >> r) & 1);
-                a[t] = inb ? M[r * ld + k] : 0.0;
-                const bool nz = inb && !is_zero_bits(a[t]);
-                l[t] = nz ? a[t] * rd : 0.0;
+                const bool inb = elim && r > k && mk.has(r);
+                const double a = inb ? Mk[r] : 0.0;
+                const bool nz = inb && !is_zero_bits(a);
+                l[t] = nz ? a * rd : 0.0;
                 const bool upd = nz && !is_zero_bits(l[t]);
                 if (act && r > k) {
                     if (upd) y[t] = fma(-l[t], yk, y[t]);
                     else {
                         // zero multiplier: zero entry times the reciprocal, or an underflow
-                        const bool neg = nz ? __double_as_longlong(l[t]) < 0 : (__double_as_longlong(a[t]) < 0) != negp;
+                        const bool neg = nz ? __double_as_longlong(l[t]) < 0 : (__double_as_longlong(a) < 0) != negp;
                         y[t] = sub_zero_product(y[t], neg, yk);
                     }
                 }
                 const unsigned b = (__ballot_sync(FULL, upd) >> q0) & gmask;
-                Lm |= (u64)b << (G * t);
+                Lm.w[G * t / 64] |= (u64)b << (G * t % 64);
             }
-            u64 rem = Lm;
-            while (__any_sync(FULL, rem != 0)) {
-                const int r = rem ? __ffsll((long long)rem) - 1 : 0;
-                const double l0 = __shfl_sync(FULL, l[0], q0 + (r & (G - 1)));
-                const double l1 = __shfl_sync(FULL, l[1], q0 + (r & (G - 1)));
-                if (rem) {
-                    const double lr = r < G ? l0 : l1;
 #pragma unroll
-                    for (int t = 0; t < 2; ++t) {
-                        const int c = g + G * t;
-                        const bool bk = (cm[t] >> k) & 1, brr = (cm[t] >> r) & 1;
-                        if (c > k && c < np && (bk || brr)) {
-                            const double mv = brr ? M[r * ld + c] : 0.0, bkv = bk ? M[k * ld + c] : 0.0;
-                            M[r * ld + c] = fma(-lr, bkv, mv);
+            for (int j = 0; j < W; ++j) {
+                u64 rem = Lm.w[j];
+                while (__any_sync(FULL, rem != 0)) {
+                    const int r = 64 * j + (rem ? __ffsll((long long)rem) - 1 : 0);
+                    double lr = 0.0;
+#pragma unroll
+                    for (int t = 0; t < R; ++t) {
+                        if (W > 1 && G * t / 64 != j) continue;
+                        const double x = __shfl_sync(FULL, l[t], q0 + (r & (G - 1)));
+                        if (r / G == t) lr = x;
+                    }
+                    if (rem) {
+#pragma unroll
+                        for (int t = 0; t < R; ++t) {
+                            const int c = g + G * t;
+                            const bool bk = cm[t].has(k), brr = cm[t].has(r);
+                            if (c > k && c < np && (bk || brr)) {
+                                double *Mc = M + (size_t)c * ld;
+                                const double mv = brr ? Mc[r] : 0.0, bkv = bk ? Mc[k] : 0.0;
+                                Mc[r] = fma(-lr, bkv, mv);
+                            }
                         }
                     }
+                    rem &= rem - 1;
                 }
-                rem &= rem - 1;
             }
 #pragma unroll
-            for (int t = 0; t < 2; ++t)
-                if (g + G * t > k && ((cm[t] >> k) & 1)) cm[t] |= Lm;
+            for (int t = 0; t < R; ++t)
+                if (g + G * t > k && cm[t].has(k)) {
+#pragma unroll
+                    for (int j = 0; j < W; ++j) cm[t].w[j] |= Lm.w[j];
+                }
             __syncwarp();
         }
         const bool solve = has && !singular && np > 0;
-        double rv[2];
+        double rv[R];
 #pragma unroll
-        for (int t = 0; t < 2; ++t) {
+        for (int t = 0; t < R; ++t) {
             const int c = g + G * t;
-            rv[t] = solve && c < np ? pivot_recip(M[c * ld + c]) : 1.0;
+            rv[t] = solve && c < np ? pivot_recip(M[(size_t)c * ld + c]) : 1.0;
         }
         for (int k = kmax - 1; k >= 0; --k) {
             const bool act = solve && k < np;
-            const u64 mk = bcast_mask(cm, k);
-            if (act && g == (k & (G - 1))) {
-                if (k < G) y[0] = times_recip(y[0], rv[0]);
-                else y[1] = times_recip(y[1], rv[1]);
-            }
+            const RowMask<W> mk = mask_column<G, R, W>(cm, k, q0);
+#pragma unroll
+            for (int t = 0; t < R; ++t)
+                if (act && g + G * t == k) y[t] = times_recip(y[t], rv[t]);
             const double yk = bcast(y, k);
             if (act)
 #pragma unroll
-                for (int t = 0; t < 2; ++t) {
+                for (int t = 0; t < R; ++t) {
                     const int r = g + G * t;
                     if (r >= k) continue;
-                    if ((mk >> r) & 1) y[t] = fma(-M[r * ld + k], yk, y[t]);
+                    if (mk.has(r)) y[t] = fma(-M[(size_t)k * ld + r], yk, y[t]);
                     else y[t] = sub_zero_product(y[t], false, yk);
                 }
         }
         long long zmb = 0;
 #pragma unroll
-        for (int t = 0; t < 2; ++t)
+        for (int t = 0; t < R; ++t)
             if (solve && g + G * t < np) zmb = max(zmb, absbits(y[t]));
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) zmb = max(zmb, __shfl_xor_sync(FULL, zmb, o, G));
@@ -1060,7 +1129,7 @@ __global__ void k_lair_solve_mask(int nwork, const int *worklist, const int *cpt
         const int base = has ? zrowptr[ic] : 0;
         int kept = 0;
 #pragma unroll
-        for (int t = 0; t < 2; ++t) {
+        for (int t = 0; t < R; ++t) {
             const int c = g + G * t;
             const bool k_ = solve && c < np && !(phi_R > 0.0 && fabs(y[t]) < thr);
             const unsigned b = (__ballot_sync(FULL, k_) >> q0) & gmask;
@@ -2001,34 +2070,38 @@ void build_hierarchy(Hier &h) {
             int *list = dmalloc<int>(nc, s);
             partition_by_class(ccls, nc, LAIR_CLASSES, list, hstart, hc, s);
             dfree(ccls, s);
-            const int cls_n[LAIR_CLASSES] = {4, 6, 8, 12, 16, 24, 32, 48, 64, 0};
-            int smem_optin = 0;
-            {
-                int dev = 0;
-                PR_CUDA(cudaGetDevice(&dev));
-                PR_CUDA(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-            }
-            auto mask_bin = [&](int c, auto kern, int G) {
+            const int cls_n[LAIR_CLASSES] = {4, 6, 8, 12, 16, 24, 32, 48, 64, 128, 256, 0};
+            // blocks of one to four warps, so that the shared memory of an SM fills evenly
+            auto mask_bin = [&](int c, auto kern, int G, int R) {
                 if (!hc[c]) return;
                 const int nm = cls_n[c], spw = 32 / G;
-                const size_t per = ((size_t)nm * (nm | 1) + nm + G) * sizeof(double) * spw;   // per warp
-                // blocks of up to four warps: many small blocks fill the SM's shared memory
-                // (and so its resident warps) evenly
-                const int wpb = (int)std::max<size_t>(1, std::min<size_t>(4, (size_t)smem_optin / per));
+                const size_t per = ((size_t)nm * (nm | 1) + nm + G * R / 2) * sizeof(double) * spw;   // per warp
+                const int wpb = per > 16 * 1024 ? 1 : per > 8 * 1024 ? 2 : 4;
                 const size_t sm = per * wpb;
                 const unsigned grid = std::min<unsigned>(blocks_for(hc[c], wpb * spw), 152u * 256u);
                 if (sm > 48 * 1024) allow_max_dyn_smem(kern);
                 kern<<<grid, 32 * wpb, sm, s>>>(hc[c], list + hstart[c], L.cpts, L.rowptr, L.col, L.val, candptr,
-                                                cand, npat, zr, zc, zv, keep, dsing, L.rowdir, prm.phi_R, nm);
+                                                cand, npat, zr, zc, zv, keep, dsing, L.rowdir, prm.phi_R, nm, nullptr);
                 PR_LAUNCH();
             };
-            for (int c = 0; c <= 2; ++c) mask_bin(c, k_lair_solve_mask<4>, 4);
-            mask_bin(3, k_lair_solve_mask<8>, 8);
-            mask_bin(4, k_lair_solve_mask<8>, 8);
-            mask_bin(5, k_lair_solve_mask<16>, 16);
-            mask_bin(6, k_lair_solve_mask<16>, 16);
-            mask_bin(7, k_lair_solve_mask<32>, 32);
-            mask_bin(8, k_lair_solve_mask<32>, 32);
+            // more than 64 unknowns: a warp a system, its workspace a slot of global memory
+            auto mask_big = [&](int c, auto kern, int R, unsigned warps) {
+                if (!hc[c]) return;
+                const int nm = cls_n[c];
+                const unsigned grid = std::min<unsigned>(hc[c], warps);
+                double *gbuf = dmalloc<double>((size_t)grid * nm * (nm | 1), s);
+                kern<<<grid, 32, ((size_t)nm + 16 * R) * sizeof(double), s>>>(
+                    hc[c], list + hstart[c], L.cpts, L.rowptr, L.col, L.val, candptr, cand, npat, zr, zc, zv, keep,
+                    dsing, L.rowdir, prm.phi_R, nm, gbuf);
+                PR_LAUNCH();
+                dfree(gbuf, s);
+            };
+            for (int c = 0; c <= 2; ++c) mask_bin(c, k_lair_solve_mask<4, 2, false>, 4, 2);
+            for (int c = 3; c <= 4; ++c) mask_bin(c, k_lair_solve_mask<8, 2, false>, 8, 2);
+            for (int c = 5; c <= 6; ++c) mask_bin(c, k_lair_solve_mask<16, 2, false>, 16, 2);
+            for (int c = 7; c <= 8; ++c) mask_bin(c, k_lair_solve_mask<32, 2, false>, 32, 2);
+            mask_big(9, k_lair_solve_mask<32, 4, true>, 4, 152u * 20u);
+            mask_big(10, k_lair_solve_mask<32, 8, true>, 8, 152u * 12u);
             int nbig = hc[LAIR_BIG];
             if (nbig > 0) {
                 long long *goff = dmalloc<long long>(nbig + 1, s);
@@ -2036,9 +2109,9 @@ void build_hierarchy(Hier &h) {
                 PR_LAUNCH();
                 const long long gtot = scan_exclusive_ll(goff, nbig, s);
                 double *gbuf = dmalloc<double>(gtot, s);
-                k_lair_solve<32><<<std::min<unsigned>(nbig, 152u * 16u), 32, 0, s>>>(
+                k_lair_solve_dense<<<std::min<unsigned>(nbig, 152u * 16u), 32, 0, s>>>(
                     nbig, list + hstart[LAIR_BIG], L.cpts, L.rowptr, L.col, L.val, candptr, cand, npat, zr, zc, zv, keep,
-                    dsing, L.rowdir, prm.phi_R, 0, goff, gbuf);
+                    dsing, L.rowdir, prm.phi_R, goff, gbuf);
                 PR_LAUNCH();
                 dfree(gbuf, s); dfree(goff, s);
             }
