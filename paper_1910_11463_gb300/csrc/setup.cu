@@ -522,65 +522,101 @@ __device__ __forceinline__ int pat_find(const int *pat, int np, int k) {
 }
 
 // ---- nAIR of degree 1 (Neumann series cut after the linear term) -----------
-// Thread per C point, on the distance-2 pattern (sorted, from k_lair_pattern):
+// On the distance-2 pattern (sorted, from k_lair_pattern2):
 //   t_k = a_ik for strong F neighbours k of i (else 0); for every strong F
-//   neighbour j of i (ascending) and every strong F neighbour k != j of j
+//   neighbour j of i (ascending) and every strong F neighbour k of j
 //   (ascending): t_k = fma(a_ij, n_jk, t_k), n_jk = -(a_jk * (1/a_jj));
 //   z_k = -(t_k * (1/a_kk)), i.e. Z_i = -A_CF^s[i,:] (I + N) D^{-1} with
 //   N = I - D^{-1} A_FF^s.  A zero diagonal on the way empties the row (counted
-//   as singular).  The values are accumulated in the row's slots of zval and the
-//   phi_R filter compacts them in place.
-__global__ void k_nair(int nc, const int *cpts, const int *rowptr, const int *col, const double *val,
-                       const uint8_t *S, const int8_t *cf, const double *dinv, const int *candptr, const int *cand,
-                       const int *npat, const int *zrowptr, int *zcol, double *zval, int *keep, int *nsing_dir,
-                       const int *rowdir, double phi_R) {
-    int ic = blockIdx.x * blockDim.x + threadIdx.x;
-    if (ic >= nc) return;
-    const int i = cpts[ic];
-    const int np = npat[ic];
-    const int *pat = cand + candptr[ic];
-    const int base = zrowptr[ic];
-    double *t = zval + base;
-    for (int e = 0; e < np; ++e) t[e] = 0.0;
-    for (int p = rowptr[i]; p < rowptr[i + 1]; ++p) {
-        int k = col[p];
-        if ((S[p] & 2) && cf[k] == CF_F) t[pat_find(pat, np, k)] = val[p];
+//   as singular).
+// Eight lanes per C row: lanes across a neighbour's row (its columns are distinct, so each
+// t_k still takes its terms in the order of j), pattern and t in shared memory up to
+// NAIR_SH unknowns, in the row's slots of cand and zval beyond.  (A thread per row that searched and
+// accumulated in global memory took 1.6 ms a level on 27^3, 8 directions.)
+constexpr int NAIR_SH = 96;
+
+__global__ void __launch_bounds__(128) k_nair(int nc, const int *cpts, const int *rowptr, const int *col,
+                                              const double *val, const uint8_t *S, const double *dinv,
+                                              const int *candptr, const int *cand, const int *npat,
+                                              const int *zrowptr, int *zcol, double *zval, int *keep, int *nsing_dir,
+                                              const int *rowdir, double phi_R) {
+    __shared__ double tsh[16][NAIR_SH];
+    __shared__ int psh[16][NAIR_SH];
+    const unsigned FULL = 0xffffffffu;
+    const int grp = threadIdx.x >> 3, lane = threadIdx.x & 31, g = lane & 7, q0 = lane & ~7;
+    const int ic = blockIdx.x * 16 + grp;
+    const bool has = ic < nc;
+    const int i = has ? cpts[ic] : 0, np = has ? npat[ic] : 0;
+    const int base = has ? zrowptr[ic] : 0;
+    const int *cp = has ? cand + candptr[ic] : nullptr;
+    const bool sh = np <= NAIR_SH;
+    double *t = sh ? tsh[grp] : zval + base;
+    const int *pat = sh ? psh[grp] : cp;
+    for (int e = g; e < np; e += 8) {
+        t[e] = 0.0;
+        if (sh) psh[grp][e] = cp[e];
     }
+    __syncwarp();
+    const int p0 = has ? rowptr[i] : 0, p1 = has ? rowptr[i + 1] : 0;
+    for (int p = p0 + g; p < p1; p += 8)
+        if (S[p] & S_RF) t[pat_find(pat, np, col[p])] = val[p];
+    __syncwarp();
     bool singular = false;
-    for (int p = rowptr[i]; p < rowptr[i + 1] && !singular; ++p) {
-        int j = col[p];
-        if (!((S[p] & 2) && cf[j] == CF_F)) continue;
-        const double aij = val[p], rj = dinv[j];
-        if (rj == 0.0) { singular = true; break; }
-        for (int q = rowptr[j]; q < rowptr[j + 1]; ++q) {
-            int k = col[q];
-            if (k == j || !((S[q] & 2) && cf[k] == CF_F)) continue;
-            const double njk = -(val[q] * rj);
-            const int e = pat_find(pat, np, k);
-            t[e] = fma(aij, njk, t[e]);
+    int len = p1 - p0;
+    for (int o = 16; o > 0; o >>= 1) len = max(len, __shfl_xor_sync(FULL, len, o));
+    for (int c0 = 0; c0 < len; c0 += 8) {
+        const int p = p0 + c0 + g;
+        const bool in = p < p1 && (S[p] & S_RF);
+        const int j = in ? col[p] : 0;
+        const double aij = in ? val[p] : 0.0, rj = in ? dinv[j] : 0.0;
+        const int js = in ? rowptr[j] : 0, je = in ? rowptr[j + 1] : 0;
+        if (in && rj == 0.0) singular = true;
+        unsigned m = (__ballot_sync(FULL, in) >> q0) & 0xffu;   // the group's neighbours of this pass
+        while (__any_sync(FULL, m != 0)) {
+            const int src = q0 + (m ? __ffs(m) - 1 : 0);
+            const double a = __shfl_sync(FULL, aij, src), r = __shfl_sync(FULL, rj, src);
+            const int s0 = __shfl_sync(FULL, js, src), s1 = __shfl_sync(FULL, je, src);
+            if (m)
+                for (int q = s0 + g; q < s1; q += 8) {
+                    if (!(S[q] & S_RF)) continue;
+                    const int e = pat_find(pat, np, col[q]);
+                    t[e] = fma(a, -(val[q] * r), t[e]);
+                }
+            __syncwarp();
+            m &= m - 1;
         }
     }
-    for (int e = 0; e < np && !singular; ++e)
+    for (int e = g; e < np; e += 8)
         if (dinv[pat[e]] == 0.0) singular = true;
-    int kept = 0;
-    if (singular) {
-        atomicAdd(&nsing_dir[rowdir[i]], 1);
-    } else {
-        long long zmb = 0;
-        for (int e = 0; e < np; ++e) {
-            t[e] = -(t[e] * dinv[pat[e]]);
-            zmb = max(zmb, absbits(t[e]));
+    singular = ((__ballot_sync(FULL, singular) >> q0) & 0xffu) != 0;
+    long long zmb = 0;
+    if (!singular)
+        for (int e = g; e < np; e += 8) {
+            const double z = -(t[e] * dinv[pat[e]]);
+            t[e] = z;
+            zmb = max(zmb, absbits(z));
         }
-        const double thr = phi_R * __longlong_as_double(zmb);
-        for (int e = 0; e < np; ++e) {
-            const double z = t[e];
-            if (phi_R > 0.0 && fabs(z) < thr) continue;
-            zcol[base + kept] = pat[e];
-            zval[base + kept] = z;
-            ++kept;
+    for (int o = 4; o > 0; o >>= 1) zmb = max(zmb, __shfl_xor_sync(FULL, zmb, o, 8));
+    const double thr = phi_R * __longlong_as_double(zmb);
+    __syncwarp();
+    int kept = 0, npm = np;
+    for (int o = 16; o > 0; o >>= 1) npm = max(npm, __shfl_xor_sync(FULL, npm, o));
+    for (int e0 = 0; e0 < npm; e0 += 8) {
+        const int e = e0 + g;
+        const double z = e < np ? t[e] : 0.0;
+        const bool k_ = e < np && !singular && !(phi_R > 0.0 && fabs(z) < thr);
+        const unsigned b = (__ballot_sync(FULL, k_) >> q0) & 0xffu;   // (t of this pass is read)
+        if (k_) {
+            const int off = base + kept + __popc(b & ((1u << g) - 1u));
+            zcol[off] = pat[e];
+            zval[off] = z;
         }
+        kept += __popc(b);
     }
-    keep[ic] = kept;
+    if (has && g == 0) {
+        if (singular) atomicAdd(&nsing_dir[rowdir[i]], 1);
+        keep[ic] = kept;
+    }
 }
 
 
@@ -2117,8 +2153,8 @@ void build_hierarchy(Hier &h) {
         int *dsing = dmalloc<int>(ND, s);
         PR_CUDA(cudaMemsetAsync(dsing, 0, sizeof(int) * ND, s));
         if (prm.nair) {
-            k_nair<<<blocks_for(nc, 128), 128, 0, s>>>(nc, L.cpts, L.rowptr, L.col, L.val, S, L.cf, L.dinv, candptr,
-                                                       cand, npat, zr, zc, zv, keep, dsing, L.rowdir, prm.phi_R);
+            k_nair<<<blocks_for(nc, 16), 128, 0, s>>>(nc, L.cpts, L.rowptr, L.col, L.val, S, L.dinv, candptr, cand, npat,
+                                                      zr, zc, zv, keep, dsing, L.rowdir, prm.phi_R);
             PR_LAUNCH();
         } else {
             // rows binned by system size; shared memory per warp sized to the bin
