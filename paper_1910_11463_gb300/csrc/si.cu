@@ -843,7 +843,7 @@ void build_batch(DirBatch &B, const pair_mesh &mesh, const double *omega_h, cons
     dd_enable(*h);
     inner_enable(*h);
     split0_enable(*h);
-    level0_bytes(*h);
+    if (timing) level0_bytes(*h);   // (only timed iterations report traffic)
     if (timing) prof_enable(*h);
 }
 
