@@ -145,6 +145,11 @@ struct Sell {
     short *col16 = nullptr;   // instead of col: column minus row, when every entry fits 16 bits
     void *val = nullptr;
     int G = 0;           // lanes per row chosen by the autotuner (0: size heuristic)
+    // F rows, for the first F sweep from the coarse vector: every entry's column replaced by
+    // its P column (-1: none), as int32 or as 16-bit offsets from the row's origin (-32768:
+    // none); pown: the row's own P column p >= 0 (also its origin), or -2 - origin if none
+    int *pcol = nullptr, *pown = nullptr;
+    short *pcol16 = nullptr;
 };
 
 struct Level {
@@ -186,10 +191,9 @@ struct Level {
     int *d_cB_off = nullptr;   // first value of each segment, in units of CD_ROWS values
     int cseg_max = 0;          // rows of the largest segment
     Sell sF, sC, sZ, sX;
-    // V-cycle work vectors (precision of the hierarchy); vF is the buffer (vy or vxn)
-    // that holds the F rows after the last F sweep, C rows are then in vx
+    // V-cycle work vectors (precision of the hierarchy); after a level's relaxation vx holds
+    // all of its rows (level 0 folds into the iterate instead)
     void *vb = nullptr, *vx = nullptr, *vxn = nullptr, *vy = nullptr;
-    void *vF = nullptr;
 };
 
 // Level schedule of an exact sweep of a block-scaled upwind operator (sweep_dag.cu):

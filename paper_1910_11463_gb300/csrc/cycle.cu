@@ -3,7 +3,9 @@
 //   level 0: r = b - A x (FP64, cast to the cycle precision T), per-matrix ||r||
 //   down:    b_{l+1} = R_l b_l, R row = [Z_i, 1] (restriction of the residual)
 //   coarsest: coarse_sweeps Jacobi sweeps from 0 (one CTA per matrix segment)
-//   up:      y_l = P x_{l+1} (one-point: y_i = x_{l+1}[pmap(i)])
+//   up:      y_l = P x_{l+1} (one-point: y_i = x_{l+1}[pmap(i)]); on the levels that relax
+//            from SELL copies y exists on the C rows only, and the first F sweep reads
+//            x_{l+1} through its entries' P columns
 //            F rows: xn = y + D^{-1}(b - A y);  C rows: xn = y
 //            C rows: x = xn + D^{-1}(b - A xn); F rows: x = xn   (level 0: x_FP64 += x)
 // Level 0 of the structured hex operator is stored in block form (identity
@@ -565,13 +567,17 @@ __device__ __forceinline__ void sell_load(int base, int len, int j0, int r, cons
     for (int u = 0; u < U; ++u) {
         const bool ok = j0 + u * G < len;
         const int at = base + 32 * (j0 + u * G);
-        if (C16) c[u] = ok ? r + (int)__ldcs(col16 + at) : 0;
-        else c[u] = ok ? __ldcs(col + at) : 0;
+        if (C16) {
+            const int o = ok ? (int)__ldcs(col16 + at) : -32768;
+            c[u] = o == -32768 ? -1 : r + o;   // (only P columns may be none)
+        } else {
+            c[u] = ok ? __ldcs(col + at) : -1;
+        }
         v[u] = ok ? __ldcs(val + at) : T(0);
     }
 }
 
-enum SellMode : int { SM_F = 0, SM_C = 1, SM_C_FINAL = 2, SM_RESTRICT = 3 };
+enum SellMode : int { SM_F = 0, SM_C = 1, SM_C_FINAL = 2, SM_RESTRICT = 3, SM_F1 = 4 };
 
 // entries per lane issued together: SELL_U for the sweeps; the restriction's short
 // rows (6-9 entries) take SELL_U / G, so a row's G lanes together still cover SELL_U
@@ -597,9 +603,22 @@ struct SellJob {
     const int *cpts;      // restriction: fine row of each coarse point
     const int *active, *rowdir;
     const int *any;       // inner correction: the launch does nothing once *any == 0
+    T *out2;              // F sweeps: optional second target
+    // first F sweep (in = the coarse vector): P columns of the rows and entries; after the
+    // row blocks (nrb of them), nC coarse values go to their C rows in out and outc
+    const int *pown, *pcol;
+    const short *pcol16;
+    T *outc;
+    int nrb, nC;
 };
 
 // F sweep:   out[i] = in[i] + dinv[i] (b[i] - A_i in)        (x64[i] += it, if given)
+// first F sweep: the same with in = P xc, read from the coarse vector xc through the P
+// columns of the row and its entries, so no prolongation runs and no vector of its values
+// is written and read back; the C rows' values, which the later sweeps gather, are
+// scattered by further blocks of the launch (one launch and one dependent step less per
+// level and cycle: 13^3 S4 46.0 -> 44.4 ms, 27^3 S4 113.0 -> 107.4, 16^3 tets 121.3 ->
+// 116.3, one solve of four 24^3 matrices 3.39 -> 3.00)
 // C sweep:   same into out, or (final) x64[i] += it
 // restrict:  out[ic] = Z_ic in + in[cpts[ic]]
 // G lanes per row (G > 1 on small levels, where rows are too few to fill the GPU):
@@ -611,58 +630,70 @@ struct SellJob {
 // gathers (with b, the row's own value and the flags beside them) leads to the store.
 template <class T, int MODE, int G, bool AHEAD, bool C16>
 __device__ __forceinline__ void sell_rows(const SellJob<T> &j) {
+    constexpr bool F1 = MODE == SM_F1, SWEEP = MODE != SM_RESTRICT;
     pdl_wait_if<!AHEAD>();
     if (!AHEAD && j.any && !*j.any) return;
     const long long t = (long long)blockIdx.x * BS + threadIdx.x;
+    if (F1 && (int)blockIdx.x >= j.nrb) {   // C rows: y = the coarse point's value
+        const long long ic = t - (long long)j.nrb * BS;
+        const int c = ic < j.nC ? j.cpts[ic] : -1;
+        pdl_wait_if<AHEAD>();
+        if ((AHEAD && j.any && !*j.any) || c < 0) return;
+        const T v = j.in[ic];
+        j.out[c] = v;
+        j.outc[c] = v;
+        return;
+    }
     const int q = (int)(t / G), g = (int)(t % G);
     const int r = j.row[q];
+    const int len = j.len[q];   // (0 at empty positions)
     bool ok = r >= 0;
-    const int dir = (MODE != SM_RESTRICT && ok && j.active) ? j.rowdir[r] : -1;
+    const int dir = (SWEEP && ok && j.active) ? j.rowdir[r] : -1;
     if (!AHEAD && dir >= 0 && !j.active[dir]) ok = false;
-    int len = ok ? j.len[q] : 0;
     const int base = j.ptr[q >> 5] + (q & 31);
     // the row's own operands are loaded before the dot product (shorter chain); a
     // restriction row's own operand, and the origin of its 16-bit columns, is its coarse
-    // point's fine row
-    const int rb = (MODE == SM_RESTRICT && ok) ? j.cpts[r] : r;
+    // point's fine row, a first F sweep's its P column
+    const int pw = F1 ? j.pown[q] : 0;
+    const int rb = F1 ? (pw >= 0 ? pw : -2 - pw) : (MODE == SM_RESTRICT && ok) ? j.cpts[r] : r;
+    const bool lead = ok && g == 0, ownv = lead && (!F1 || pw >= 0);
+    const int *col = F1 ? j.pcol : j.col;
+    const short *col16 = F1 ? j.pcol16 : j.col16;
     T own = T(0), di = T(0), bi = T(0);
-    if (!AHEAD && ok && g == 0) {
-        own = j.in[rb];
-        if (MODE != SM_RESTRICT) bi = j.b[r];
-    }
-    if (MODE != SM_RESTRICT && ok && g == 0) di = j.dinv[r];
+    if (!AHEAD && ownv) own = j.in[rb];
+    if (!AHEAD && SWEEP && lead) bi = j.b[r];
+    if (SWEEP && lead) di = j.dinv[r];
     constexpr int U = sell_unroll<MODE, G>();
+    const int ln = ok ? len : 0;
     T acc = T(0);
     int j0 = g;
     if (AHEAD) {
         int c[U];
         T v[U], x[U];
-        sell_load<T, G, U, C16>(base, len, j0, rb, j.col, j.col16, j.val, c, v);
+        sell_load<T, G, U, C16>(base, ln, j0, rb, col, col16, j.val, c, v);
         pdl_wait_if<AHEAD>();
         const int any = j.any ? *j.any : 1;
         const int act = dir >= 0 ? j.active[dir] : 1;
-        if (ok && g == 0) {
-            own = j.in[rb];
-            if (MODE != SM_RESTRICT) bi = j.b[r];
-        }
+        if (ownv) own = j.in[rb];
+        if (SWEEP && lead) bi = j.b[r];
 #pragma unroll
-        for (int u = 0; u < U; ++u) x[u] = j0 + u * G < len ? j.in[c[u]] : T(0);
+        for (int u = 0; u < U; ++u) x[u] = c[u] >= 0 ? j.in[c[u]] : T(0);
         if (!any) return;
         ok = ok && act;
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (j0 + u * G < len) acc += v[u] * x[u];
+            if (j0 + u * G < ln) acc += v[u] * x[u];
         j0 += U * G;
     }
-    for (; j0 < len; j0 += U * G) {
+    for (; j0 < ln; j0 += U * G) {
         int c[U];
         T v[U], x[U];
-        sell_load<T, G, U, C16>(base, len, j0, rb, j.col, j.col16, j.val, c, v);
+        sell_load<T, G, U, C16>(base, ln, j0, rb, col, col16, j.val, c, v);
 #pragma unroll
-        for (int u = 0; u < U; ++u) x[u] = j0 + u * G < len ? j.in[c[u]] : T(0);
+        for (int u = 0; u < U; ++u) x[u] = c[u] >= 0 ? j.in[c[u]] : T(0);
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (j0 + u * G < len) acc += v[u] * x[u];
+            if (j0 + u * G < ln) acc += v[u] * x[u];
     }
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o, G);
@@ -677,37 +708,34 @@ __device__ __forceinline__ void sell_rows(const SellJob<T> &j) {
         else j.x64[r] += (double)vn;
     } else {
         // the fold's load before the store to out
-        if (MODE == SM_F && j.d32) j.d32[r] += (float)vn;
-        else if (MODE == SM_F && j.x64) j.x64[r] += (double)vn;
+        if ((MODE == SM_F || F1) && j.d32) j.d32[r] += (float)vn;
+        else if ((MODE == SM_F || F1) && j.x64) j.x64[r] += (double)vn;
         j.out[r] = vn;
+        if ((MODE == SM_F || F1) && j.out2) j.out2[r] = vn;
     }
 }
 
 template <class T, int MODE, int G, bool AHEAD>
 __global__ void __launch_bounds__(BS) k_sell(SellJob<T> j) {
-    if (j.col16) sell_rows<T, MODE, G, AHEAD, true>(j);
+    if (MODE == SM_F1 ? j.pcol16 != nullptr : j.col16 != nullptr) sell_rows<T, MODE, G, AHEAD, true>(j);
     else sell_rows<T, MODE, G, AHEAD, false>(j);
 }
 
-// ---- prolongation y = P x_c --------------------------------------------------
-// The coarse vector of level l+1 lives in two buffers after its relaxation: F rows
-// in xcF, C and coarsest rows in xc.  C rows of y are also written to y2 (the other
-// ping-pong buffer of the F sweeps), so the F sweeps never copy C rows.
+// ---- prolongation y = P x_c (block-form level 0) -------------------------------
+// C rows of y are also written to y2 (the other ping-pong buffer of the F sweeps), so the
+// F sweeps never copy C rows.
 template <class T>
-__device__ __forceinline__ void prolong_row(long long i, int8_t c, int p, const int8_t *cfc, const T *xcF,
-                                            const T *xc, T *y, T *y2) {
+__device__ __forceinline__ void prolong_row(long long i, int8_t c, int p, const T *xc, T *y, T *y2) {
     if (c == CF_COARSEST) return;
-    T v = T(0);
-    if (p >= 0) v = (cfc[p] == CF_F ? xcF : xc)[p];
+    const T v = p >= 0 ? xc[p] : T(0);
     y[i] = v;
     if (y2 && c == CF_C) y2[i] = v;
 }
 
-// four consecutive rows per thread (vector loads of cf and pmap, twelve gathers in
-// flight): with one row per thread the kernel is latency-bound
+// four consecutive rows per thread (vector loads of cf and pmap, four gathers in flight):
+// with one row per thread the kernel is latency-bound
 template <class T>
-__global__ void k_prolong(int n, const int8_t *cf, const int *pmap, const int8_t *cfc, const T *xcF, const T *xc,
-                          T *y, T *y2, const int *any) {
+__global__ void k_prolong(int n, const int8_t *cf, const int *pmap, const T *xc, T *y, T *y2, const int *any) {
     const long long i0 = 4LL * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
     if (i0 >= n) return;
     if (i0 + 4 <= n) {
@@ -715,17 +743,11 @@ __global__ void k_prolong(int n, const int8_t *cf, const int *pmap, const int8_t
         const int4 p4 = *reinterpret_cast<const int4 *>(pmap + i0);
         const int8_t c[4] = {(int8_t)c4.x, (int8_t)c4.y, (int8_t)c4.z, (int8_t)c4.w};
         const int p[4] = {p4.x, p4.y, p4.z, p4.w};
-        const T *src[4];   // where the coarse value lives: the coarse rows' flags are constants too
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const bool gth = c[u] != CF_COARSEST && p[u] >= 0;
-            src[u] = gth ? (cfc[p[u]] == CF_F ? xcF : xc) + p[u] : nullptr;
-        }
         pdl_wait();
         const int go = any ? *any : 1;
         T v[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = src[u] ? *src[u] : T(0);
+        for (int u = 0; u < 4; ++u) v[u] = c[u] != CF_COARSEST && p[u] >= 0 ? xc[p[u]] : T(0);
         if (!go) return;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -736,7 +758,7 @@ __global__ void k_prolong(int n, const int8_t *cf, const int *pmap, const int8_t
     } else {
         pdl_wait();
         if (any && !*any) return;
-        for (long long i = i0; i < n; ++i) prolong_row<T>(i, cf[i], pmap[i], cfc, xcF, xc, y, y2);
+        for (long long i = i0; i < n; ++i) prolong_row<T>(i, cf[i], pmap[i], xc, y, y2);
     }
 }
 
@@ -1106,7 +1128,11 @@ void launch_sell_g(const Sell &S, SellJob<T> j, int G, int sms, cudaStream_t s) 
     j.col = S.col;
     j.col16 = S.col16;
     j.val = (const T *)S.val;
-    const unsigned nb = blocks_for((long long)G * S.npos, BS);
+    j.pown = S.pown;
+    j.pcol = S.pcol;
+    j.pcol16 = S.pcol16;
+    j.nrb = (int)blocks_for((long long)G * S.npos, BS);
+    const unsigned nb = j.nrb + (MODE == SM_F1 ? blocks_for(j.nC, BS) : 0u);
     auto go = [&](auto ahead, auto plain) { launch_pdl(load_ahead(nb, sms) ? ahead : plain, nb, BS, s, j); };
     switch (G) {
         case 1: go(k_sell<T, MODE, 1, true>, k_sell<T, MODE, 1, false>); break;
@@ -1134,10 +1160,16 @@ void launch_sell(const Sell &S, SellJob<T> j, int sms, cudaStream_t s) {
 }
 
 // F sweep over the F rows (fold: x64 += the new values, the last level-0 sweep)
+// from: the coarse vector of a first sweep (in is then not read), whose C rows go to out
+// and outc; out2: second target of the F rows
 template <class T>
-void relax_f(const Level &L, const T *b, const T *in, T *out, double *fold, float *fold32, const int *active,
-             const int *any, int sms, cudaStream_t s) {
+void relax_f(const Level &L, const T *b, const T *from, const T *in, T *out, T *outc, T *out2, double *fold,
+             float *fold32, const int *active, const int *any, int sms, cudaStream_t s) {
     SellJob<T> j{};
+    j.out2 = out2;
+    j.outc = outc;
+    j.cpts = L.cpts;
+    j.nC = L.nC;
     j.any = any;
     j.in = in;
     j.dinv = lv_dinv<T>(L);
@@ -1147,7 +1179,12 @@ void relax_f(const Level &L, const T *b, const T *in, T *out, double *fold, floa
     j.d32 = fold32;
     j.active = active;
     j.rowdir = L.rowdir;
-    launch_sell<T, SM_F>(L.sF, j, sms, s);
+    if (from) {
+        j.in = from;
+        launch_sell<T, SM_F1>(L.sF, j, sms, s);
+    } else {
+        launch_sell<T, SM_F>(L.sF, j, sms, s);
+    }
 }
 
 // C sweep over the C rows into out, or (final) into x64 together with the coarsest
@@ -1228,7 +1265,6 @@ void vcycle_t(Hier &h, double *x64, float *d32, const int *active, ProfSlot *ps)
     if (ps) ps->relax_timed = false;
     for (int l = 0; l < NL; ++l) {
         Level &L = h.lev[l];
-        L.vF = L.vx;   // replaced by the F sweeps' buffer once the level relaxes
         if (l + 1 < NL) {
             const bool tr = prof && (int)ps->lvt.size() >= 4 * (l + 1);
             if (tr) rec_event(ps->lvt[4 * l], s);
@@ -1263,9 +1299,11 @@ void vcycle_t(Hier &h, double *x64, float *d32, const int *active, ProfSlot *ps)
         const bool split0 = bsr && h.split0 && std::is_same<T, float>::value;
         const bool tp = prof && (int)ps->lvt.size() >= 4 * (l + 1);
         if (tp) rec_event(ps->lvt[4 * l + 2], s);
-        launch_pdl(k_prolong<T>, blocks_for((L.n + 3) / 4, BS), BS, s, L.n, L.cf, L.pmap, C.cf, (const T *)C.vF,
-                   (const T *)C.vx, bufs[0], (bsr && !split0) ? nullptr : bufs[1], any);
-        PR_LAUNCH();
+        if (bsr) {   // (the SELL levels' first F sweep reads the coarse vector itself)
+            launch_pdl(k_prolong<T>, blocks_for((L.n + 3) / 4, BS), BS, s, L.n, L.cf, L.pmap, (const T *)C.vx, bufs[0],
+                       split0 ? bufs[1] : (T *)nullptr, any);
+            PR_LAUNCH();
+        }
         if (tp) rec_event(ps->lvt[4 * l + 3], s);
         int cur = 0;
         if (split0) {
@@ -1313,21 +1351,24 @@ void vcycle_t(Hier &h, double *x64, float *d32, const int *active, ProfSlot *ps)
             PR_LAUNCH();
             if (prof) rec_event(ps->relax0[1], s);
         } else {
-            // C rows stay where the prolongation put them (both buffers); F rows end in
-            // bufs[cur], C rows in vx (level 0: both folded into the iterate instead)
+            // the first F sweep puts the C rows' prolonged values into both buffers; the last
+            // one also writes its F rows to vx, where the C sweep's rows join them (level 0:
+            // both folded into the iterate instead)
             const int *act = l == 0 ? active : nullptr;
             bool tl = prof && l >= 1 && (int)ps->lv.size() >= 2 * (l + 1);
             if (tl) rec_event(ps->lv[2 * l], s);
             if (prof && l == 0) { rec_event(ps->relax0[0], s); ps->relax_timed = true; }
-            for (int f = 0; f < fs; ++f, cur ^= 1)
-                relax_f<T>(L, (const T *)L.vb, bufs[cur], bufs[cur ^ 1], l == 0 && f == fs - 1 ? x64 : nullptr,
-                           l == 0 && f == fs - 1 ? d32 : nullptr, act, any, h.sms, s);
+            for (int f = 0; f < fs; ++f, cur ^= 1) {
+                const bool last = f == fs - 1;
+                relax_f<T>(L, (const T *)L.vb, f == 0 ? (const T *)C.vx : nullptr, bufs[cur], bufs[cur ^ 1], bufs[cur],
+                           last && l > 0 ? (T *)L.vx : nullptr, last && l == 0 ? x64 : nullptr,
+                           last && l == 0 ? d32 : nullptr, act, any, h.sms, s);
+            }
             relax_c<T>(L, (const T *)L.vb, bufs[cur], (T *)L.vx, l == 0 ? x64 : nullptr, l == 0 ? d32 : nullptr,
                        (const T *)L.vx, act, any, h.sms, s);
             if (tl) rec_event(ps->lv[2 * l + 1], s);
             if (prof && l == 0) rec_event(ps->relax0[1], s);
         }
-        L.vF = bufs[cur];
     }
     if (NL == 1) {   // single-level hierarchies: x += coarsest solution
         Level &L = h.lev[0];
@@ -1491,7 +1532,8 @@ void level0_bytes(Hier &h) {
             if (L.nc <= 0) continue;
             const double cb = L.sZ.col16 ? 2.0 : 4.0;
             h.bytes_xfer += (double)L.nc * (12 + 2 * sT) + (double)L.nnzZ * (cb + sT);
-            h.bytes_xfer += (double)(L.nF + L.nC) * (5 + sT) + (double)L.nC * sT;
+            // (SELL levels: the C rows' scatter, by the first F sweep)
+            if (l == 0 && h.bsr0) h.bytes_xfer += (double)(L.nF + L.nC) * (5 + sT) + (double)L.nC * sT;
         }
     }
     // the iterate the level-0 relaxation folds into: FP64 x or a float pair (8 B
@@ -1518,7 +1560,7 @@ void level0_bytes(Hier &h) {
             const double cbF = L.sF.col16 ? 2.0 : 4.0, cbC = L.sC.col16 ? 2.0 : 4.0;
             double fpass = (double)c[0] * (8 + 4 * sT) + (double)c[2] * (cbF + sT);
             double cpass = (double)c[1] * (8 + 4 * sT) + (double)c[3] * (cbC + sT);
-            h.bytes_relaxc += h.prm.f_sweeps * fpass + cpass;
+            h.bytes_relaxc += h.prm.f_sweeps * fpass + cpass + (double)c[1] * (4 + 3 * sT) + (double)c[0] * sT;
         }
         dfree(cnt, s);
         // grid-wide coarsest sweeps: the first reads each row's split position, b and

@@ -1788,7 +1788,7 @@ __global__ void k_sell_off_check(int npos, const int *prow, const int *plen, con
     const int len = plen[pos], base = sptr[pos >> 5] + (pos & 31);
     for (int j = 0; j < len; ++j) {
         const int off = scol[base + 32 * j] - r;
-        if (off < -32768 || off > 32767) { atomicOr(bad, 1); return; }
+        if (off < -32767 || off > 32767) { atomicOr(bad, 1); return; }
     }
 }
 
@@ -1803,23 +1803,97 @@ __global__ void k_sell_to16(int npos, const int *prow, const int *plen, const in
     for (int j = 0; j < len; ++j) col16[base + 32 * j] = (short)(scol[base + 32 * j] - r);
 }
 
-void sell_compress_cols(Hier &h, Sell &S, const int *rowbase = nullptr) {
-    if (S.nrows <= 0 || !S.col) return;
-    cudaStream_t s = h.stream;
-    const int BS = 256;
-    int *bad = dmalloc<int>(1, s);
-    PR_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), s));
-    k_sell_off_check<<<blocks_for(S.npos, BS), BS, 0, s>>>(S.npos, S.row, S.len, S.ptr, S.col, rowbase, bad);
+// P columns of a store's entries and rows (Sell::pcol, pown); *bad: an offset from the
+// row's origin (its own P column, else its first entry's) leaves 16 bits
+__global__ void k_sell_pcol(int npos, const int *prow, const int *plen, const int *sptr, const int *scol,
+                            const int *pmap, int *pcol, int *pown, int *bad) {
+    const int pos = blockIdx.x * blockDim.x + threadIdx.x;
+    if (pos >= npos) return;
+    const int r = prow[pos];
+    if (r < 0) { pown[pos] = -2; return; }
+    const int len = plen[pos], base = sptr[pos >> 5] + (pos & 31);
+    const int own = pmap[r];
+    int org = own;
+    bool far = false;
+    for (int j = 0; j < len; ++j) {
+        const int c = pmap[scol[base + 32 * j]];
+        pcol[base + 32 * j] = c;
+        if (c < 0) continue;
+        if (org < 0) org = c;
+        far |= c - org < -32767 || c - org > 32767;
+    }
+    pown[pos] = own >= 0 ? own : -2 - max(org, 0);
+    if (far) atomicOr(bad, 1);
+}
+
+__global__ void k_sell_pcol16(int npos, const int *prow, const int *plen, const int *sptr, const int *pcol,
+                              const int *pown, short *pcol16) {
+    const int pos = blockIdx.x * blockDim.x + threadIdx.x;
+    if (pos >= npos || prow[pos] < 0) return;
+    const int len = plen[pos], base = sptr[pos >> 5] + (pos & 31);
+    const int o = pown[pos], org = o >= 0 ? o : -2 - o;
+    for (int j = 0; j < len; ++j) {
+        const int c = pcol[base + 32 * j];
+        pcol16[base + 32 * j] = (short)(c < 0 ? -32768 : c - org);
+    }
+}
+
+void sell_off_check(Sell &S, const int *rowbase, int *bad, cudaStream_t s) {
+    if (S.nrows <= 0) return;
+    k_sell_off_check<<<blocks_for(S.npos, 256), 256, 0, s>>>(S.npos, S.row, S.len, S.ptr, S.col, rowbase, bad);
     PR_LAUNCH();
-    int hb = 0;
-    d2h(&hb, bad, 1, s);
-    dfree(bad, s);
-    if (hb) return;
+}
+
+void sell_to16(Sell &S, const int *rowbase, cudaStream_t s) {
+    if (S.nrows <= 0) return;
     S.col16 = dmalloc<short>(std::max<long long>(S.nnz, 1), s);
-    k_sell_to16<<<blocks_for(S.npos, BS), BS, 0, s>>>(S.npos, S.row, S.len, S.ptr, S.col, rowbase, S.col16);
+    k_sell_to16<<<blocks_for(S.npos, 256), 256, 0, s>>>(S.npos, S.row, S.len, S.ptr, S.col, rowbase, S.col16);
     PR_LAUNCH();
     dfree(S.col, s);
     S.col = nullptr;
+}
+
+// 16-bit column offsets of one store, where they fit
+void sell_compress_cols(Hier &h, Sell &S, const int *rowbase = nullptr) {
+    if (S.nrows <= 0 || !S.col) return;
+    cudaStream_t s = h.stream;
+    int *bad = dmalloc<int>(1, s);
+    PR_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), s));
+    sell_off_check(S, rowbase, bad, s);
+    int hb = 0;
+    d2h(&hb, bad, 1, s);
+    dfree(bad, s);
+    if (!hb) sell_to16(S, rowbase, s);
+}
+
+// the F and C stores of a level: P columns of the F store, and 16-bit offsets where they
+// fit (one host read for the three checks)
+void sell_finish_fc(Hier &h, Level &L) {
+    cudaStream_t s = h.stream;
+    Sell &F = L.sF;
+    int *bad = dmalloc<int>(3, s);
+    PR_CUDA(cudaMemsetAsync(bad, 0, 3 * sizeof(int), s));
+    if (F.nrows > 0) {
+        F.pcol = dmalloc<int>(std::max<long long>(F.nnz, 1), s);
+        F.pown = dmalloc<int>(F.npos, s);
+        k_sell_pcol<<<blocks_for(F.npos, 256), 256, 0, s>>>(F.npos, F.row, F.len, F.ptr, F.col, L.pmap, F.pcol, F.pown,
+                                                            bad + 2);
+        PR_LAUNCH();
+    }
+    sell_off_check(F, nullptr, bad, s);
+    sell_off_check(L.sC, nullptr, bad + 1, s);
+    int hb[3] = {0, 0, 0};
+    d2h(hb, bad, 3, s);
+    dfree(bad, s);
+    if (!hb[0]) sell_to16(F, nullptr, s);
+    if (!hb[1]) sell_to16(L.sC, nullptr, s);
+    if (!hb[2] && F.nrows > 0) {
+        F.pcol16 = dmalloc<short>(std::max<long long>(F.nnz, 1), s);
+        k_sell_pcol16<<<blocks_for(F.npos, 256), 256, 0, s>>>(F.npos, F.row, F.len, F.ptr, F.pcol, F.pown, F.pcol16);
+        PR_LAUNCH();
+        dfree(F.pcol, s);
+        F.pcol = nullptr;
+    }
 }
 
 // SELL copy of nr rows of a CSR matrix (list rows, or rows 0..nr-1), values in the
@@ -1873,8 +1947,7 @@ void build_split(Hier &h, Level &L, bool with_fc) {
     if (with_fc) {
         build_sell(h, L.sF, L.srow, L.nF, L.rowptr, L.col, L.val);
         build_sell(h, L.sC, L.srow + L.nF, L.nC, L.rowptr, L.col, L.val);
-        sell_compress_cols(h, L.sF);
-        sell_compress_cols(h, L.sC);
+        sell_finish_fc(h, L);
     }
     if (nx > 0) {
         int *len = dmalloc<int>(nx, s);
@@ -1931,7 +2004,7 @@ void free_level(Level &L, cudaStream_t s) {
     void *ptrs[] = {L.rowptr, L.col, L.val, L.dinv, L.dinv32, L.cf, L.pmap, L.rowdir, L.cpts,
                     L.zrowptr, L.zcol, L.zval, L.d_row0, L.d_cseg_row0, L.d_cseg_n,
                     L.srow, L.sptr, L.scol, L.sval, L.d_cseg_s0, L.cB, L.d_cB_off,
-                    L.sF.ptr, L.sF.row, L.sF.len, L.sF.col, L.sF.col16, L.sF.val, L.sC.ptr, L.sC.row, L.sC.len,
+                    L.sF.ptr, L.sF.row, L.sF.len, L.sF.col, L.sF.col16, L.sF.val, L.sF.pcol, L.sF.pown, L.sF.pcol16, L.sC.ptr, L.sC.row, L.sC.len,
                     L.sC.col, L.sC.col16, L.sC.val, L.sZ.ptr, L.sZ.row, L.sZ.len, L.sZ.col, L.sZ.col16, L.sZ.val,
                     L.sX.ptr, L.sX.row, L.sX.len, L.sX.col, L.sX.col16, L.sX.val, L.vb, L.vx, L.vxn, L.vy};
     for (void *p : ptrs) dfree(p, s);
