@@ -145,15 +145,22 @@ __device__ __forceinline__ void for_strong(int i, const int *rowptr, const uint8
 __global__ void k_pmis_init(int n, const int *rowdir, const char *dwork, const int *row0, const unsigned *lam,
                             int level, unsigned long long seed, uint64_t *key, int8_t *state, int *undecided) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int d = rowdir[i];
-    if (!dwork[d]) { state[i] = ST_F; key[i] = 0; return; }
-    uint64_t li = (uint64_t)(i - row0[d]);
-    uint32_t hh = (uint32_t)(splitmix_first(seed ^ ((uint64_t)level << 40) ^ li) >> 32);
-    key[i] = ((uint64_t)lam[i] << 32) | hh;
-    int8_t s = lam[i] == 0 ? ST_F : ST_U;
-    state[i] = s;
-    if (s == ST_U) atomicAdd(undecided, 1);
+    int8_t s = ST_F;
+    if (i < n) {
+        int d = rowdir[i];
+        if (!dwork[d]) {
+            key[i] = 0;
+        } else {
+            uint64_t li = (uint64_t)(i - row0[d]);
+            uint32_t hh = (uint32_t)(splitmix_first(seed ^ ((uint64_t)level << 40) ^ li) >> 32);
+            key[i] = ((uint64_t)lam[i] << 32) | hh;
+            if (lam[i] != 0) s = ST_U;
+        }
+        state[i] = s;
+    }
+    // one atomic per block: they all meet at one address
+    const int c = __syncthreads_count(s == ST_U);
+    if (threadIdx.x == 0 && c) atomicAdd(undecided, c);
 }
 
 __device__ __forceinline__ bool key_gt(uint64_t kj, int j, uint64_t ki, int i) {
@@ -178,18 +185,21 @@ __global__ void k_pmis_mark(int n, const int *rowptr, const int *col, const uint
 __global__ void k_pmis_update(int n, const int *rowptr, const int *col, const uint8_t *S, const unsigned *smask,
                               const int8_t *state, int8_t *next, const int *notmax, int round, int *undecided) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int8_t s = state[i];
-    if (s != ST_U) { next[i] = s; return; }
-    if (notmax[i] != round) { next[i] = ST_C; return; }
-    bool f = false;
-    for_strong(i, rowptr, S, smask, [&](int p) {
-        const int j = col[p];
-        f = state[j] == ST_U && notmax[j] != round;
-        return !f;
-    });
-    next[i] = f ? ST_F : ST_U;
-    if (!f) atomicAdd(undecided, 1);
+    int8_t s = i < n ? state[i] : ST_F;
+    if (s == ST_U) {
+        if (notmax[i] != round) {
+            s = ST_C;
+        } else {
+            for_strong(i, rowptr, S, smask, [&](int p) {
+                const int j = col[p];
+                if (state[j] == ST_U && notmax[j] != round) s = ST_F;
+                return s == ST_U;
+            });
+        }
+    }
+    if (i < n) next[i] = s;
+    const int c = __syncthreads_count(s == ST_U);
+    if (threadIdx.x == 0 && c) atomicAdd(undecided, c);
 }
 
 // per-matrix sums: one atomic per warp when its rows share a matrix (the usual case)
@@ -271,26 +281,42 @@ __global__ void k_mark_rf(int n, const int *rowptr, const int *col, const int8_t
     if (i < n && g == 0) nf[i] = c;
 }
 
-// Candidates (with repeats) of every C row.  Rows with more than PAT_BIG of them go to
-// the list of the bitmap kernel (any order: a row's pattern has its own place).
-constexpr int PAT_SMALL = 64, PAT_MID = 256, PAT_BIG = 1024;
-
-__global__ void k_lair_ncand(int nc, const int *cpts, const int *rowptr, const int *col, const uint8_t *S,
-                             const int *nf, int distance, int *ncand, int *big, int *nbig) {
+// distance 1: the C rows alone are marked and counted (their marked entries are the
+// pattern)
+__global__ void k_mark_rf1(int nc, const int *cpts, const int *rowptr, const int *col, const int8_t *cf, uint8_t *S,
+                           int *ncand) {
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int ic = (int)(tid >> 3), g = (int)(tid & 7);
     int c = 0;
     if (ic < nc) {
         const int i = cpts[ic];
-        if (distance < 2) c = g == 0 ? nf[i] : 0;
-        else
-            for (int p = rowptr[i] + g; p < rowptr[i + 1]; p += 8)
-                if (S[p] & S_RF) c += 1 + nf[col[p]];
+        for (int p = rowptr[i] + g; p < rowptr[i + 1]; p += 8) {
+            const uint8_t f = S[p];
+            if ((f & 2) && cf[col[p]] == CF_F) { S[p] = f | S_RF; ++c; }
+        }
+    }
+    for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if (ic < nc && g == 0) ncand[ic] = c;
+}
+
+// distance 2: candidates (with repeats) of every C row.  Rows with more than PAT_BIG of them go to
+// the list of the bitmap kernel (any order: a row's pattern has its own place).
+constexpr int PAT_SMALL = 64, PAT_MID = 256, PAT_BIG = 1024;
+
+__global__ void k_lair_ncand(int nc, const int *cpts, const int *rowptr, const int *col, const uint8_t *S,
+                             const int *nf, int *ncand, int *big, int *nbig) {
+    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int ic = (int)(tid >> 3), g = (int)(tid & 7);
+    int c = 0;
+    if (ic < nc) {
+        const int i = cpts[ic];
+        for (int p = rowptr[i] + g; p < rowptr[i + 1]; p += 8)
+            if (S[p] & S_RF) c += 1 + nf[col[p]];
     }
     for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if (ic < nc && g == 0) {
         ncand[ic] = c;
-        if (distance >= 2 && c > PAT_BIG) big[atomicAdd(nbig, 1)] = ic;
+        if (c > PAT_BIG) big[atomicAdd(nbig, 1)] = ic;
     }
 }
 
@@ -1056,6 +1082,17 @@ __global__ void k_lair_solve_mask(int nwork, const int *worklist, const int *cpt
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) kmax = max(kmax, __shfl_xor_sync(FULL, kmax, o));
         const long long tinyb = absbits(1e-14 * __longlong_as_double(mxb));
+        // reciprocals of the diagonal as gathered, all at once: a division holds the FP64 pipe
+        // for a hundred cycles and more however few lanes take part, and most rows reach
+        // their pivot step unchanged, so one per step and one per row again at the end was
+        // much of the pipe's work on the levels without a unit diagonal
+        double d0[R], rv[R];
+#pragma unroll
+        for (int t = 0; t < R; ++t) {
+            const int c = g + G * t;
+            d0[t] = c < np && cm[t].has(c) ? M[(size_t)c * ld + c] : 1.0;
+            rv[t] = pivot_recip(d0[t]);
+        }
         bool singular = false;
         for (int k = 0; k < kmax; ++k) {
             bool act = k < np && !singular;
@@ -1125,10 +1162,15 @@ __global__ void k_lair_solve_mask(int nwork, const int *worklist, const int *cpt
                         if (g + G * t > k) y[t] = sub_zero_product(y[t], negp, yk);
                 continue;
             }
-            // the pivot's reciprocal: one lane of the group divides
-            double rd = 0.0;
-            if (elim && g == 0) rd = pivot_recip(pk);
-            rd = __shfl_sync(FULL, rd, q0);
+            // the pivot's reciprocal: one lane of the group divides if the pivot has changed
+            double rd = bcast(rv, k);
+            const double dk = bcast(d0, k);   // (every lane takes part in the broadcasts)
+            const bool redo = elim && __double_as_longlong(pk) != __double_as_longlong(dk);
+            if (__any_sync(FULL, redo)) {
+                double r1 = rd;
+                if (redo && g == 0) r1 = pivot_recip(pk);
+                rd = __shfl_sync(FULL, r1, q0);
+            }
             RowMask<W> Lm;   // rows whose multiplier is not zero
 #pragma unroll
             for (int j = 0; j < W; ++j) Lm.w[j] = 0;
@@ -1188,11 +1230,11 @@ __global__ void k_lair_solve_mask(int nwork, const int *worklist, const int *cpt
             __syncwarp();
         }
         const bool solve = has && !singular && np > 0;
-        double rv[R];
 #pragma unroll
         for (int t = 0; t < R; ++t) {
             const int c = g + G * t;
-            rv[t] = solve && c < np ? pivot_recip(M[(size_t)c * ld + c]) : 1.0;
+            const double p = solve && c < np ? M[(size_t)c * ld + c] : d0[t];
+            if (__double_as_longlong(p) != __double_as_longlong(d0[t])) rv[t] = pivot_recip(p);
         }
         for (int k = kmax - 1; k >= 0; --k) {
             const bool act = solve && k < np;
@@ -2179,25 +2221,30 @@ void build_hierarchy(Hier &h) {
         // ---- lAIR -----------------------------------------------------------
         const int rdist = prm.nair ? 2 : prm.distance;   // nAIR degree 1 uses the distance-2 pattern
         int *ncand = dmalloc<int>(nc, s);
-        int *nf = dmalloc<int>(n, s);
-        k_mark_rf<<<blocks_for(8LL * n, BS), BS, 0, s>>>(n, L.rowptr, L.col, L.cf, S, nf);
-        PR_LAUNCH();
-        int *pbig = dmalloc<int>(rdist >= 2 ? nc + 1 : 1, s);   // [count, rows with many candidates]
-        PR_CUDA(cudaMemsetAsync(pbig, 0, sizeof(int), s));
-        k_lair_ncand<<<blocks_for(8LL * nc, BS), BS, 0, s>>>(nc, L.cpts, L.rowptr, L.col, S, nf, rdist, ncand,
-                                                             pbig + 1, pbig);
-        PR_LAUNCH();
-        dfree(nf, s);
+        int *pbig = nullptr;   // distance 2: [count, rows with many candidates]
+        if (rdist < 2) {
+            k_mark_rf1<<<blocks_for(8LL * nc, BS), BS, 0, s>>>(nc, L.cpts, L.rowptr, L.col, L.cf, S, ncand);
+            PR_LAUNCH();
+        } else {
+            int *nf = dmalloc<int>(n, s);
+            k_mark_rf<<<blocks_for(8LL * n, BS), BS, 0, s>>>(n, L.rowptr, L.col, L.cf, S, nf);
+            PR_LAUNCH();
+            pbig = dmalloc<int>((size_t)nc + 1, s);
+            PR_CUDA(cudaMemsetAsync(pbig, 0, sizeof(int), s));
+            k_lair_ncand<<<blocks_for(8LL * nc, BS), BS, 0, s>>>(nc, L.cpts, L.rowptr, L.col, S, nf, ncand, pbig + 1,
+                                                                 pbig);
+            PR_LAUNCH();
+            dfree(nf, s);
+        }
         int *candptr = dmalloc<int>(nc + 1, s);
         long long ncandt = scan_exclusive(ncand, candptr, nc, s);
         int *cand = dmalloc<int>(ncandt, s);
         int *npat = ncand;   // distance 1: the candidates are the pattern
-        int *zr = dmalloc<int>(nc + 1, s);
+        int *zr = candptr;     // and their offsets the rows of Z
         long long nz = ncandt;
         if (rdist < 2) {
             k_lair_pattern1<<<blocks_for(8LL * nc, BS), BS, 0, s>>>(nc, L.cpts, L.rowptr, L.col, S, candptr, cand);
             PR_LAUNCH();
-            PR_CUDA(cudaMemcpyAsync(zr, candptr, sizeof(int) * (nc + 1), cudaMemcpyDeviceToDevice, s));
         } else {
             // one launch per size class over all rows (a row of another class costs its
             // count), no partition and no host read
@@ -2217,6 +2264,7 @@ void build_hierarchy(Hier &h) {
                                                                                  L.col, S, candptr, cand, npat);
             PR_LAUNCH();
             dfree(ncand, s);
+            zr = dmalloc<int>(nc + 1, s);
             nz = scan_exclusive(npat, zr, nc, s);
         }
         dfree(pbig, s);
@@ -2294,11 +2342,10 @@ void build_hierarchy(Hier &h) {
             double *zv2 = dmalloc<double>(nz2, s);
             k_compact_rows<<<blocks_for(8LL * nc, BS), BS, 0, s>>>(nc, zr, zr2, zc, zv, zc2, zv2);
             PR_LAUNCH();
-            dfree(zc, s); dfree(zv, s); dfree(zr, s);
+            dfree(zc, s); dfree(zv, s);
             zc = zc2; zv = zv2;
-        } else {
-            dfree(zr, s);
         }
+        if (zr != candptr) dfree(zr, s);
         L.zrowptr = zr2; L.zcol = zc; L.zval = zv; L.nnzZ = nz2;
         dfree(keep, s); dfree(cand, s); dfree(candptr, s); dfree(npat, s);
         dfree(S, s);
