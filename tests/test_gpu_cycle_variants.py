@@ -62,3 +62,33 @@ def test_coarsest_product_equals_sweeps(pair, n, sweeps):
         x = x.cpu().numpy()
         assert np.array_equal(x[:n], x[n:])
         assert np.linalg.norm(x[:n] - want) <= tol * max(np.linalg.norm(want), 1e-300)
+
+
+# the first F sweep through P columns: offsets that fit 16 bits and ones that do not, rows
+# without a coarse neighbour, one to three F sweeps; FP64 cycles of a few dozen additions a
+# row agree to 1e-12
+@pytest.mark.parametrize("n,far,f_sweeps", [(300, False, 1), (3000, False, 2), (3000, False, 3), (150_000, True, 2),
+                                            (150_000, True, 1)])
+def test_first_sweep_through_p_columns(pair, n, far, f_sweeps):
+    from oracle import oracle as O
+    g = np.random.default_rng(n + f_sweeps)
+    k = 3
+    off = g.integers(0, n, (n, k)) if far else np.clip(np.arange(n)[:, None] + g.integers(-20, 21, (n, k)), 0, n - 1)
+    off[::9] = np.arange(n)[::9, None]   # rows that depend on nothing
+    rows = np.repeat(np.arange(n), k)
+    cols = off.ravel()
+    keep = cols != rows
+    key = np.unique(rows[keep].astype(np.int64) * n + cols[keep])
+    key = np.unique(np.concatenate([key, np.arange(n, dtype=np.int64) * (n + 1)]))
+    r, c = key // n, (key % n).astype(np.int32)
+    v = np.where(r == c, 1.0, g.uniform(-0.3, 0.3, key.size))
+    rp = np.concatenate([[0], np.cumsum(np.bincount(r, minlength=n))]).astype(np.int32)
+    kw = dict(theta=0.5, max_coarse=50, max_levels=4, f_sweeps=f_sweeps)
+    b, x0 = g.random(n), g.random(n)
+    h = pair.Hierarchy([tuple(torch.as_tensor(a, device="cuda") for a in (rp, c, v))],
+                       pair.default_air_params(precision=0, **kw))
+    x = h.vcycle(torch.as_tensor(b, device="cuda"), torch.as_tensor(x0, device="cuda").clone()).cpu().numpy()
+    H = O.Hierarchy(rp, c, v, O.default_params(**kw))
+    assert H.nlev >= 2
+    xo = H.vcycle(b, x0.copy())
+    assert np.linalg.norm(x - xo) <= 1e-12 * np.linalg.norm(xo)
