@@ -390,11 +390,11 @@ pair_status dg_assemble_tet(const pair_mesh *mesh, const double *omega, const do
         PR_CUDA(cudaMemcpyAsync(om, omega, 3 * sizeof(double), cudaMemcpyHostToDevice, s));
         PR_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
         long long z = pr::tet_assemble(mesh->ntet, 1, om, mesh->verts, mesh->tets, mesh->nbr, sigma_t, rowptr,
-                                       nullptr, nullptr, nullptr, nullptr, err, s, true);
+                                       nullptr, nullptr, nullptr, nullptr, err, s, pr::TET_ROWPTR);
         *nnz = (int)z;
         if (col && val && capacity >= z)
             pr::tet_assemble(mesh->ntet, 1, om, mesh->verts, mesh->tets, mesh->nbr, sigma_t, rowptr, col, val,
-                             nullptr, nullptr, err, s, false);
+                             nullptr, nullptr, err, s, pr::TET_VALUES);
         int herr = 0;
         PR_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
         PR_CUDA(cudaStreamSynchronize(s));

@@ -20,41 +20,8 @@ namespace {
 
 // LU with partial pivoting (first maximum), multipliers a_rk * (1 / a_kk),
 // updates fma(-l, a_kc, a_rc); column-oriented substitutions with fma and
-// y_k * (1 / u_kk).  The same operation sequence as every LU in the library.
-template <int n>
-__device__ __forceinline__ void lu_factorN(double *a, int *piv, double *rinv, int *singular) {
-    for (int k = 0; k < n; ++k) {
-        int p = k;
-        long long mx = absbits(a[k * n + k]);
-        for (int r = k + 1; r < n; ++r) {
-            long long v = absbits(a[r * n + k]);
-            if (v > mx) { mx = v; p = r; }
-        }
-        piv[k] = p;
-        if (!(mx > 0)) { *singular = 1; return; }
-        if (p != k)
-            for (int c = 0; c < n; ++c) { double t = a[k * n + c]; a[k * n + c] = a[p * n + c]; a[p * n + c] = t; }
-        double rd = 1.0 / a[k * n + k];
-        rinv[k] = rd;   // row k is final from here on: the back substitution reuses it
-        for (int r = k + 1; r < n; ++r) {
-            double l = a[r * n + k] * rd;
-            a[r * n + k] = l;
-            for (int c = k + 1; c < n; ++c) a[r * n + c] = fma(-l, a[k * n + c], a[r * n + c]);
-        }
-    }
-}
-
-template <int n>
-__device__ __forceinline__ void lu_solveN(const double *a, const int *piv, const double *rinv, double *y) {
-    for (int k = 0; k < n; ++k)
-        if (piv[k] != k) { double t = y[k]; y[k] = y[piv[k]]; y[piv[k]] = t; }
-    for (int k = 0; k < n; ++k)
-        for (int r = k + 1; r < n; ++r) y[r] = fma(-a[r * n + k], y[k], y[r]);
-    for (int k = n - 1; k >= 0; --k) {
-        y[k] = y[k] * rinv[k];
-        for (int r = 0; r < k; ++r) y[r] = fma(-a[r * n + k], y[k], y[r]);
-    }
-}
+// y_k * (1 / u_kk).  The same operation sequence as every LU in the library
+// (lu_step, lu_solve below).
 
 struct HexFactors {
     double m1[2][2];
@@ -98,67 +65,68 @@ constexpr int HA_BS = 128;
 
 // step K of the factorisation (a template, so that every loop bound and index is a
 // constant and D stays in registers)
-template <int K>
-__device__ __forceinline__ void lu8_step(double (&D)[64], int (&piv)[8], double (&rinv)[8], int &singular) {
+template <int N, int K = 0>
+__device__ __forceinline__ void lu_step(double (&D)[N * N], int (&piv)[N], double (&rinv)[N], int &singular) {
     int p = K;
-    long long mx = absbits(D[K * 8 + K]);
+    long long mx = absbits(D[K * N + K]);
 #pragma unroll
-    for (int r = K + 1; r < 8; ++r) {
-        const long long v = absbits(D[r * 8 + K]);
+    for (int r = K + 1; r < N; ++r) {
+        const long long v = absbits(D[r * N + K]);
         if (v > mx) { mx = v; p = r; }
     }
     piv[K] = p;
     if (!(mx > 0)) singular = 1;
     if (p != K) {
 #pragma unroll
-        for (int r = K + 1; r < 8; ++r)
+        for (int r = K + 1; r < N; ++r)
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const double u = D[K * 8 + c], v = D[r * 8 + c];
-                D[K * 8 + c] = p == r ? v : u;
-                D[r * 8 + c] = p == r ? u : v;
+            for (int c = 0; c < N; ++c) {
+                const double u = D[K * N + c], v = D[r * N + c];
+                D[K * N + c] = p == r ? v : u;
+                D[r * N + c] = p == r ? u : v;
             }
     }
-    const double rd = 1.0 / D[K * 8 + K];
+    const double rd = 1.0 / D[K * N + K];
     rinv[K] = rd;   // row K is final from here on: the back substitution reuses it
 #pragma unroll
-    for (int r = K + 1; r < 8; ++r) {
-        const double l = D[r * 8 + K] * rd;
-        D[r * 8 + K] = l;
+    for (int r = K + 1; r < N; ++r) {
+        const double l = D[r * N + K] * rd;
+        D[r * N + K] = l;
 #pragma unroll
-        for (int c = K + 1; c < 8; ++c) D[r * 8 + c] = fma(-l, D[K * 8 + c], D[r * 8 + c]);
+        for (int c = K + 1; c < N; ++c) D[r * N + c] = fma(-l, D[K * N + c], D[r * N + c]);
     }
-    if constexpr (K < 7) lu8_step<K + 1>(D, piv, rinv, singular);
+    if constexpr (K < N - 1) lu_step<N, K + 1>(D, piv, rinv, singular);
 }
 
-template <int K>
-__device__ __forceinline__ void lu8_swap(const int (&piv)[8], double (&y)[8]) {
+template <int N, int K = 0>
+__device__ __forceinline__ void lu_swap(const int (&piv)[N], double (&y)[N]) {
 #pragma unroll
-    for (int r = K + 1; r < 8; ++r) {
+    for (int r = K + 1; r < N; ++r) {
         const double u = y[K], v = y[r];
         y[K] = piv[K] == r ? v : u;
         y[r] = piv[K] == r ? u : v;
     }
-    if constexpr (K < 6) lu8_swap<K + 1>(piv, y);
+    if constexpr (K < N - 2) lu_swap<N, K + 1>(piv, y);
 }
-template <int K>
-__device__ __forceinline__ void lu8_fwd(const double (&D)[64], double (&y)[8]) {
+template <int N, int K = 0>
+__device__ __forceinline__ void lu_fwd(const double (&D)[N * N], double (&y)[N]) {
 #pragma unroll
-    for (int r = K + 1; r < 8; ++r) y[r] = fma(-D[r * 8 + K], y[K], y[r]);
-    if constexpr (K < 6) lu8_fwd<K + 1>(D, y);
+    for (int r = K + 1; r < N; ++r) y[r] = fma(-D[r * N + K], y[K], y[r]);
+    if constexpr (K < N - 2) lu_fwd<N, K + 1>(D, y);
 }
-template <int K>
-__device__ __forceinline__ void lu8_bwd(const double (&D)[64], const double (&rinv)[8], double (&y)[8]) {
+template <int N, int K = N - 1>
+__device__ __forceinline__ void lu_bwd(const double (&D)[N * N], const double (&rinv)[N], double (&y)[N]) {
     y[K] = y[K] * rinv[K];
 #pragma unroll
-    for (int r = 0; r < K; ++r) y[r] = fma(-D[r * 8 + K], y[K], y[r]);
-    if constexpr (K > 0) lu8_bwd<K - 1>(D, rinv, y);
+    for (int r = 0; r < K; ++r) y[r] = fma(-D[r * N + K], y[K], y[r]);
+    if constexpr (K > 0) lu_bwd<N, K - 1>(D, rinv, y);
 }
-__device__ __forceinline__ void lu8_solve(const double (&D)[64], const int (&piv)[8], const double (&rinv)[8],
-                                          double (&y)[8]) {
-    lu8_swap<0>(piv, y);
-    lu8_fwd<0>(D, y);
-    lu8_bwd<7>(D, rinv, y);
+template <int N>
+__device__ __forceinline__ void lu_solve(const double (&D)[N * N], const int (&piv)[N], const double (&rinv)[N],
+                                         double (&y)[N]) {
+    lu_swap<N>(piv, y);
+    lu_fwd<N>(D, y);
+    lu_bwd<N>(D, rinv, y);
 }
 
 __global__ void __launch_bounds__(HA_BS) k_hex_assemble(int n, const double *omega, const double *sigma_t,
@@ -223,7 +191,7 @@ __global__ void __launch_bounds__(HA_BS) k_hex_assemble(int n, const double *ome
     int piv[8];
     double rinv[8];
     int sing = 0;
-    lu8_step<0>(D, piv, rinv, sing);
+    lu_step<8>(D, piv, rinv, sing);
     if (sing && has) atomicOr(err, 1);   // (the host stops before anything reads the rows)
 
     const int idx[3] = {e % n, (e / n) % n, e / (n * n)};
@@ -263,7 +231,7 @@ __global__ void __launch_bounds__(HA_BS) k_hex_assemble(int n, const double *ome
             double y[8];
 #pragma unroll
             for (int a = 0; a < 8; ++a) y[a] = fin[d][t][a];
-            lu8_solve(D, piv, rinv, y);
+            lu_solve<8>(D, piv, rinv, y);
 #pragma unroll
             for (int a = 0; a < 8; ++a) sg[lane][a * 4 + t] = up[d] ? y[a] : 0.0;
         }
@@ -306,7 +274,7 @@ __global__ void __launch_bounds__(HA_BS) k_hex_assemble(int n, const double *ome
             }
             y[a] = acc;
         }
-        lu8_solve(D, piv, rinv, y);
+        lu_solve<8>(D, piv, rinv, y);
         if (has)
 #pragma unroll
             for (int a = 0; a < 8; ++a) Gin[((long long)m * E + e) * 8 + a] = y[a];
@@ -320,7 +288,7 @@ __global__ void __launch_bounds__(HA_BS) k_hex_assemble(int n, const double *ome
                 double y[8];
 #pragma unroll
                 for (int a = 0; a < 8; ++a) y[a] = mass[a * 8 + b];
-                lu8_solve(D, piv, rinv, y);
+                lu_solve<8>(D, piv, rinv, y);
 #pragma unroll
                 for (int a = 0; a < 8; ++a) sg[lane][a * 4 + t] = y[a];
             }
@@ -343,10 +311,10 @@ __global__ void __launch_bounds__(HA_BS) k_hex_assemble(int n, const double *ome
 // face flux (Omega.n)|F| = -(od_f (3 |K|)).
 // L_KK[a][b] = sigma_t (c_ab |K| / 20) - (od_a |K|) / 4 + sum_{outflow f, a,b != f} (fl_f c_ab) / 12
 // L_KK'[a][b'] = (fl_f c) / 12 on the inflow face f (c = 2 on the same vertex, else 1).
-struct TetGeom {
-    double od[4], fl[4], vol;
-};
-
+// What a tet's geometry alone fixes (the gradients and |K|) is formed once per tet by
+// k_tet_geom and read back for every direction: its ten divisions were most of the FP64
+// work of an element, again for each of the 24 or 80 directions and again for the row
+// counts.
 __device__ __forceinline__ void cross3(const double *a, const double *b, double *c) {
     c[0] = a[1] * b[2] - a[2] * b[1];
     c[1] = a[2] * b[0] - a[0] * b[2];
@@ -354,7 +322,13 @@ __device__ __forceinline__ void cross3(const double *a, const double *b, double 
 }
 __device__ __forceinline__ double dot3(const double *a, const double *b) { return (a[0] * b[0] + a[1] * b[1]) + a[2] * b[2]; }
 
-__device__ __forceinline__ bool tet_geom(const double *verts, const int *tv, const double *om, TetGeom &g) {
+// geometry, one array of T per component: gradients (4 x 3), then |K| (-1: zero volume)
+constexpr int TET_GEOM = 13;
+
+__global__ void k_tet_geom(int T, const double *verts, const int *tets, double *geom) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= T) return;
+    const int *tv = tets + 4LL * t;
     double x[4][3], e[3][3], gr[4][3], c23[3], c31[3], c12[3];
     for (int a = 0; a < 4; ++a)
         for (int k = 0; k < 3; ++k) x[a][k] = verts[3 * tv[a] + k];
@@ -363,36 +337,56 @@ __device__ __forceinline__ bool tet_geom(const double *verts, const int *tv, con
     cross3(e[1], e[2], c23);
     cross3(e[2], e[0], c31);
     cross3(e[0], e[1], c12);
-    double det = dot3(e[0], c23);
-    if (det == 0.0) return false;
+    const double det = dot3(e[0], c23);
+    if (det == 0.0) { geom[(TET_GEOM - 1LL) * T + t] = -1.0; return; }
     for (int k = 0; k < 3; ++k) {
         gr[1][k] = c23[k] / det;
         gr[2][k] = c31[k] / det;
         gr[3][k] = c12[k] / det;
         gr[0][k] = -((gr[1][k] + gr[2][k]) + gr[3][k]);
     }
-    g.vol = fabs(det) / 6.0;
-    for (int a = 0; a < 4; ++a) g.od[a] = dot3(om, gr[a]);
+    for (int a = 0; a < 4; ++a)
+        for (int k = 0; k < 3; ++k) geom[(3LL * a + k) * T + t] = gr[a][k];
+    geom[(TET_GEOM - 1LL) * T + t] = fabs(det) / 6.0;
+}
+
+struct TetGeom {
+    double od[4], fl[4], vol;
+};
+
+__device__ __forceinline__ bool tet_geom(const double *geom, int T, int t, const double *om, TetGeom &g) {
+    g.vol = geom[(TET_GEOM - 1LL) * T + t];
+    if (g.vol == -1.0) return false;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        const double gr[3] = {geom[(3LL * a) * T + t], geom[(3LL * a + 1) * T + t], geom[(3LL * a + 2) * T + t]};
+        g.od[a] = dot3(om, gr);
+    }
+#pragma unroll
     for (int f = 0; f < 4; ++f) g.fl[f] = -(g.od[f] * (3.0 * g.vol));
     return true;
 }
 
-__global__ void k_tet_rowcounts(int T, int ndir, const double *omega, const double *verts, const int *tets,
-                                const int *nbr, int *counts) {
+__global__ void k_tet_rowcounts(int T, int ndir, const double *omega, const double *geom, const int *nbr, int *counts) {
     long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (tid >= (long long)T * ndir) return;
     int m = (int)(tid / T), t = (int)(tid % T);
     const double om[3] = {omega[3 * m], omega[3 * m + 1], omega[3 * m + 2]};
     TetGeom g;
     int c = 1;
-    if (tet_geom(verts, tets + 4 * t, om, g))
+    if (tet_geom(geom, T, t, om, g))
         for (int f = 0; f < 4; ++f)
-            if (g.fl[f] < 0.0 && nbr[4 * t + f] >= 0) c += 3;
-    long long r0 = ((long long)m * T + t) * 4;
-    for (int a = 0; a < 4; ++a) counts[r0 + a] = c;
+            if (g.fl[f] < 0.0 && nbr[4LL * t + f] >= 0) c += 3;
+    *reinterpret_cast<int4 *>(counts + ((long long)m * T + t) * 4) = make_int4(c, c, c, c);
 }
 
-__global__ void __launch_bounds__(128) k_tet_assemble(int T, int ndir, const double *omega, const double *verts,
+// Thread per (tet, direction); the factors in registers, each solved column stored at once.
+// FP64-pipe bound.  40^3 x 6 tets, 24 directions, row counts and assembly: 40^3 S4 solve
+// 471 -> 454 ms, 20^3 exact sweeps 23.3 -> 20.5 ms against a geometry per (tet, direction)
+// and a division per matrix entry.
+// (2 x and 1 x |K| / 20, flux / 12 differ by an exact factor of two, so each takes one
+// division.)
+__global__ void __launch_bounds__(128) k_tet_assemble(int T, int ndir, const double *omega, const double *geom,
                                                       const int *tets, const int *nbr, const double *sigma_t,
                                                       const int *rowptr, int *col, double *val, double *W,
                                                       double *Gin, int *err) {
@@ -400,98 +394,116 @@ __global__ void __launch_bounds__(128) k_tet_assemble(int T, int ndir, const dou
     if (tid >= (long long)T * ndir) return;
     int m = (int)(tid / T), t = (int)(tid % T);
     const double om[3] = {omega[3 * m], omega[3 * m + 1], omega[3 * m + 2]};
-    const int *tv = tets + 4 * t;
     TetGeom g;
-    if (!tet_geom(verts, tv, om, g)) { atomicOr(err, 1); return; }
-    double st = sigma_t[t], vol = g.vol;
+    if (!tet_geom(geom, T, t, om, g)) { atomicOr(err, 1); return; }
+    const int4 tv4 = *reinterpret_cast<const int4 *>(tets + 4LL * t);
+    const int4 nb4 = *reinterpret_cast<const int4 *>(nbr + 4LL * t);
+    const int tv[4] = {tv4.x, tv4.y, tv4.z, tv4.w}, nb[4] = {nb4.x, nb4.y, nb4.z, nb4.w};
+    const double st = sigma_t[t];
+    const double ms1 = g.vol / 20.0, ms2 = 2.0 * ms1;   // mass entries off and on the diagonal
+    double f1[4];                                       // face entries: flux / 12, twice that on the diagonal
+#pragma unroll
+    for (int f = 0; f < 4; ++f) f1[f] = g.fl[f] / 12.0;
     double D[16];
+#pragma unroll
     for (int a = 0; a < 4; ++a)
+#pragma unroll
         for (int b = 0; b < 4; ++b) {
-            double mass = ((a == b) ? 2.0 : 1.0) * vol / 20.0;
-            double v = st * mass - g.od[a] * vol / 4.0;
-            for (int f = 0; f < 4; ++f) {
-                if (!(g.fl[f] > 0.0) || a == f || b == f) continue;
-                v = v + g.fl[f] * ((a == b) ? 2.0 : 1.0) / 12.0;
-            }
+            double v = st * (a == b ? ms2 : ms1) - g.od[a] * g.vol / 4.0;
+#pragma unroll
+            for (int f = 0; f < 4; ++f)
+                if (g.fl[f] > 0.0 && a != f && b != f) v = v + (a == b ? 2.0 * f1[f] : f1[f]);
             D[a * 4 + b] = v;
         }
     int piv[4], sing = 0;
     double rinv[4];
-    lu_factorN<4>(D, piv, rinv, &sing);
+    lu_step<4>(D, piv, rinv, sing);
     if (sing) { atomicOr(err, 1); return; }
-    // inflow faces with an upwind neighbour, sorted by neighbour index with t itself
-    int nb_e[5], nb_f[5], cnt = 0;
-    for (int f = 0; f < 4; ++f)
-        if (g.fl[f] < 0.0 && nbr[4 * t + f] >= 0) { nb_e[cnt] = nbr[4 * t + f]; nb_f[cnt] = f; ++cnt; }
-    nb_e[cnt] = t;
-    nb_f[cnt] = -1;
-    int tot = cnt + 1;
-    for (int i = 1; i < tot; ++i)
-        for (int j = i; j > 0 && nb_e[j - 1] > nb_e[j]; --j) {
-            int x = nb_e[j]; nb_e[j] = nb_e[j - 1]; nb_e[j - 1] = x;
-            x = nb_f[j]; nb_f[j] = nb_f[j - 1]; nb_f[j - 1] = x;
+    const long long N = 4LL * T;
+    const long long rowbase = (long long)m * N + 4LL * t;
+    // an entry's place in its row: upwind tets and the tet itself by index
+    bool up[4];
+    int len = 1, self = 0;
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+        up[f] = g.fl[f] < 0.0 && nb[f] >= 0;
+        if (up[f]) {
+            len += 3;
+            if (nb[f] <= t) self += 3;
         }
-    double Y[4][3][4];   // [face][face node][row]
-    int Ynode[4][3];
-    for (int k = 0; k < tot; ++k) {
-        int f = nb_f[k];
-        if (f < 0) continue;
-        const int *uv = tets + 4 * nb_e[k];
+    }
+    const int rp = col ? rowptr[rowbase] : 0;   // the tet's rows are equally long
+    if (col)
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            col[rp + a * len + self] = (int)(rowbase + a);
+            val[rp + a * len + self] = 1.0;
+        }
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+        if (!up[f]) continue;
+        int off = nb[f] > t ? 1 : 0;
+#pragma unroll
+        for (int h = 0; h < 4; ++h)
+            if (h != f && up[h] && (nb[h] < nb[f] || (nb[h] == nb[f] && h < f))) off += 3;
+        const int4 u4 = *reinterpret_cast<const int4 *>(tets + 4LL * nb[f]);
+        const int uv[4] = {u4.x, u4.y, u4.z, u4.w};
         int u = 0;
-        for (int b = 0; b < 4 && u < 3; ++b) {
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
             bool onface = false;
-            for (int a = 0; a < 4; ++a)
-                if (a != f && tv[a] == uv[b]) onface = true;
-            if (!onface) continue;
-            Ynode[f][u] = b;
-            double *y = Y[f][u];
-            for (int a = 0; a < 4; ++a) y[a] = (a == f) ? 0.0 : g.fl[f] * ((tv[a] == uv[b]) ? 2.0 : 1.0) / 12.0;
-            lu_solveN<4>(D, piv, rinv, y);
+#pragma unroll
+            for (int a = 0; a < 4; ++a) onface |= a != f && tv[a] == uv[b];
+            if (!onface || u >= 3) continue;
+            double y[4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) y[a] = a == f ? 0.0 : tv[a] == uv[b] ? 2.0 * f1[f] : f1[f];
+            lu_solve<4>(D, piv, rinv, y);
+            if (col)
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    col[rp + a * len + off + u] = (int)((long long)m * N + 4LL * nb[f] + b);
+                    val[rp + a * len + off + u] = y[a];
+                }
             ++u;
         }
         if (u != 3) atomicOr(err, 2);
     }
-    long long N = 4LL * T;
-    long long rowbase = (long long)m * N + 4LL * t;
-    if (col) {
-        for (int a = 0; a < 4; ++a) {
-            long long p = rowptr[rowbase + a];
-            for (int k = 0; k < tot; ++k) {
-                int f = nb_f[k];
-                if (f < 0) { col[p] = (int)(rowbase + a); val[p] = 1.0; ++p; continue; }
-                for (int u = 0; u < 3; ++u) {
-                    col[p] = (int)((long long)m * N + 4LL * nb_e[k] + Ynode[f][u]);
-                    val[p] = Y[f][u][a];
-                    ++p;
-                }
-            }
-        }
-    }
     if (Gin) {
         // D^{-1} (boundary inflow faces: sum_b |fl_f| c_ab / 12, unit inflow)
         double y[4];
+#pragma unroll
         for (int a = 0; a < 4; ++a) {
             double acc = 0.0;
+#pragma unroll
             for (int f = 0; f < 4; ++f) {
-                if (!(g.fl[f] < 0.0) || nbr[4 * t + f] >= 0 || a == f) continue;
+                if (!(g.fl[f] < 0.0) || nb[f] >= 0 || a == f) continue;
                 double s2 = 0.0;
+#pragma unroll
                 for (int b = 0; b < 4; ++b)
-                    if (b != f) s2 = s2 + -(g.fl[f] * ((a == b) ? 2.0 : 1.0) / 12.0);
+                    if (b != f) s2 = s2 + -(a == b ? 2.0 * f1[f] : f1[f]);
                 acc = acc + s2;
             }
             y[a] = acc;
         }
-        lu_solveN<4>(D, piv, rinv, y);
+        lu_solve<4>(D, piv, rinv, y);
+#pragma unroll
         for (int a = 0; a < 4; ++a) Gin[((long long)m * T + t) * 4 + a] = y[a];
     }
     if (W) {
         double *We = W + ((long long)m * T + t) * 16;
+        double w[16];
+#pragma unroll
         for (int b = 0; b < 4; ++b) {
             double y[4];
-            for (int a = 0; a < 4; ++a) y[a] = ((a == b) ? 2.0 : 1.0) * vol / 20.0;
-            lu_solveN<4>(D, piv, rinv, y);
-            for (int a = 0; a < 4; ++a) We[a * 4 + b] = y[a];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) y[a] = a == b ? ms2 : ms1;
+            lu_solve<4>(D, piv, rinv, y);
+#pragma unroll
+            for (int a = 0; a < 4; ++a) w[a * 4 + b] = y[a];
         }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) reinterpret_cast<double2 *>(We)[q] = make_double2(w[2 * q], w[2 * q + 1]);
     }
 }
 
@@ -519,21 +531,42 @@ void hex_assemble(int n, int ndir, const double *omega_d, const double *sigma_t,
 }
 
 // Tetrahedral mesh, 'ndir' directions: CSR (rows/cols offset by m * 4T), W
-// [dir][tet][4][4] = D^{-1} M, Gin [dir][4T].  Computes rowptr; returns nnz.
+// [dir][tet][4][4] = D^{-1} M, Gin [dir][4T].  TET_ROWPTR computes the row pointer and
+// returns nnz; TET_VALUES assembles on a row pointer it computed (returns 0).
 long long tet_assemble(int T, int ndir, const double *omega_d, const double *verts, const int *tets, const int *nbr,
                        const double *sigma_t, int *rowptr, int *col, double *val, double *W, double *Gin, int *d_err,
-                       cudaStream_t s, bool rowptr_only) {
+                       cudaStream_t s, TetPass pass) {
     long long rows = 4LL * T * ndir;
     PR_REQUIRE(rows < 0x7fffffffLL, PAIR_ERR_UNSUPPORTED, "tet batch has more than 2^31 rows");
-    int *counts = dmalloc<int>(rows, s);
-    k_tet_rowcounts<<<blocks_for((long long)T * ndir, 256), 256, 0, s>>>(T, ndir, omega_d, verts, tets, nbr, counts);
+    // the kernels read tets and nbr as int4: caller arrays that are not 16-byte aligned are
+    // copied first
+    int *ctets = nullptr, *cnbr = nullptr;
+    auto aligned = [&](const int *p, int *&copy) -> const int * {
+        if (reinterpret_cast<uintptr_t>(p) % 16 == 0) return p;
+        copy = dmalloc<int>(4LL * T, s);
+        PR_CUDA(cudaMemcpyAsync(copy, p, sizeof(int) * 4LL * T, cudaMemcpyDeviceToDevice, s));
+        return copy;
+    };
+    const int *at = pass == TET_VALUES ? aligned(tets, ctets) : tets;
+    const int *an = pass == TET_VALUES ? aligned(nbr, cnbr) : nbr;
+    double *geom = dmalloc<double>((size_t)TET_GEOM * T, s);
+    k_tet_geom<<<blocks_for(T, 128), 128, 0, s>>>(T, verts, at, geom);
     PR_LAUNCH();
-    long long nnz = scan_exclusive(counts, rowptr, (int)rows, s);
-    dfree(counts, s);
-    if (rowptr_only) return nnz;
-    k_tet_assemble<<<blocks_for((long long)T * ndir, 128), 128, 0, s>>>(T, ndir, omega_d, verts, tets, nbr, sigma_t,
-                                                                        rowptr, col, val, W, Gin, d_err);
-    PR_LAUNCH();
+    long long nnz = 0;
+    if (pass == TET_ROWPTR) {
+        int *counts = dmalloc<int>(rows, s);
+        k_tet_rowcounts<<<blocks_for((long long)T * ndir, 256), 256, 0, s>>>(T, ndir, omega_d, geom, an, counts);
+        PR_LAUNCH();
+        nnz = scan_exclusive(counts, rowptr, (int)rows, s);
+        dfree(counts, s);
+    } else {
+        k_tet_assemble<<<blocks_for((long long)T * ndir, 128), 128, 0, s>>>(T, ndir, omega_d, geom, at, an, sigma_t,
+                                                                            rowptr, col, val, W, Gin, d_err);
+        PR_LAUNCH();
+    }
+    dfree(geom, s);
+    dfree(ctets, s);
+    dfree(cnbr, s);
     return nnz;
 }
 

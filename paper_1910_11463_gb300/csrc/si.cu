@@ -785,7 +785,7 @@ void build_batch(DirBatch &B, const pair_mesh &mesh, const double *omega_h, cons
     L.rowptr = dmalloc<int>(L.n + 1, s);
     if (!hex)   // entry count depends on the sign of Omega.n on every face
         nnz = tet_assemble(mesh.ntet, nd, omega_d + 3 * B.m0, mesh.verts, mesh.tets, mesh.nbr, sigma_t, L.rowptr,
-                           nullptr, nullptr, nullptr, nullptr, h->d_err, s, true);
+                           nullptr, nullptr, nullptr, nullptr, h->d_err, s, TET_ROWPTR);
     PR_REQUIRE(nnz < 0x7fffffffLL, PAIR_ERR_UNSUPPORTED, "direction batch exceeds 2^31 stored entries");
     L.nnz = nnz;
     L.col = dmalloc<int>(nnz, s);
@@ -816,7 +816,7 @@ void build_batch(DirBatch &B, const pair_mesh &mesh, const double *omega_h, cons
                      h->d_err, s);
     else
         tet_assemble(mesh.ntet, nd, omega_d + 3 * B.m0, mesh.verts, mesh.tets, mesh.nbr, sigma_t, L.rowptr, L.col,
-                     L.val, B.W, B.Gin, h->d_err, s, false);
+                     L.val, B.W, B.Gin, h->d_err, s, TET_VALUES);
     {   // an element that failed left its rows unwritten: stop before anything reads them
         int aerr = 0;
         PR_CUDA(cudaMemcpyAsync(&aerr, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));

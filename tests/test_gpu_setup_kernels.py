@@ -123,3 +123,22 @@ def test_lair_solver_bins(pair, entries, distance, phi_R):
     unknowns) that need pivoting."""
     rp, ci, va = _coupled(500, entries, 60 + entries)
     _check(pair, rp, ci, va, distance=distance, theta=0.6, phi_R=phi_R, max_levels=2, max_coarse=10)
+
+
+def test_tet_assembly_of_unaligned_index_arrays(pair):
+    """Vertex and neighbour ids that do not start on 16 bytes give the same operator."""
+    from paper_1910_11463_gb300 import inputs as I
+    prob = I.small_tet(3, order=2, seed=4)
+    st = torch.as_tensor(prob.sigma_t, device="cuda")
+    mesh = pair.TetMesh(prob.verts, prob.tets, prob.nbr)
+    want = pair.dg_assemble_tet(mesh, prob.omega[1], st)
+    moved = pair.TetMesh(prob.verts, prob.tets, prob.nbr)
+    keep = []
+    for name, a in (("tets", prob.tets), ("nbr", prob.nbr)):
+        buf = torch.zeros(a.size + 1, dtype=torch.int32, device="cuda")
+        buf[1:] = torch.as_tensor(np.ascontiguousarray(a, np.int32), device="cuda").reshape(-1)
+        keep.append(buf)
+        setattr(moved.struct, name, buf.data_ptr() + 4)
+    got = pair.dg_assemble_tet(moved, prob.omega[1], st)
+    for x, y in zip(want, got):
+        assert torch.equal(x, y)
