@@ -64,9 +64,10 @@ typedef struct pair_hier_s *pair_hier;
  *  phi_A         filter applied to every coarse operator, diagonal kept (0 = off)
  *  max_levels    level cap (including the finest)
  *  max_coarse    a level with at most this many rows is the coarsest
- *  coarse_sweeps pointwise Jacobi sweeps from zero on the coarsest level (one CTA
- *                per matrix in shared memory while a matrix's coarsest level fits
- *                40 KB; larger coarsest levels sweep grid-wide, one launch per sweep)
+ *  coarse_sweeps pointwise Jacobi sweeps from zero on the coarsest level (coarsest
+ *                levels of at most 128 rows per matrix apply them as one dense product
+ *                formed in the setup; up to 40 KB they run in one CTA per matrix in
+ *                shared memory, larger ones grid-wide, one launch per sweep)
  *  seed          PMIS key hash seed
  *  precision     0: hierarchy values and V-cycle in FP64;
  *                1: FP32 hierarchy and V-cycle under FP64 iterative refinement
@@ -331,7 +332,9 @@ typedef struct {
     int timed_iters;         /* SI iterations whose cycles the kernel timings cover
                               * (si_params.timing) */
     double t_xfer_ms;        /* grid transfers: every level's restriction (R_l applied to
-                              * b_l) and one-point prolongation, all cycles */
+                              * b_l) and the one-point prolongation to a block-form level
+                              * 0, all cycles (on the other levels the prolongation is part
+                              * of the first F sweep and counts with the relaxation) */
     int n_xfer;              /* cycles measured */
     double gb_xfer;          /* algorithmic GB of those transfers */
 } si_info;
