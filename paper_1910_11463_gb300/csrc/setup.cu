@@ -1325,7 +1325,7 @@ __global__ void __launch_bounds__(128) k_ap(int n, const int *rowptr, const int 
         int len = 0;
         if (cf[k] == CF_COARSEST) {
             aplen[k] = 0;
-        } else if (e > E || e - s > AP_SHORT) {
+        } else if (e > s && (e > E || e - s > AP_SHORT)) {   // (an empty row has no product: aplen 0 below)
             longrow[atomicAdd(nlong, 1)] = k;
         } else {
             for (int p = s; p < e; ++p) {   // slot s + len <= p: the merge runs in place

@@ -142,3 +142,27 @@ def test_tet_assembly_of_unaligned_index_arrays(pair):
     got = pair.dg_assemble_tet(moved, prob.omega[1], st)
     for x, y in zip(want, got):
         assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("distance,nair", [(1, 0), (2, 0), (1, 1)])
+def test_rows_without_entries(pair, distance, nair):
+    """A matrix whose blocks of 128 rows hold more entries than a block of the A P kernel
+    stages, with rows that hold none: some of those are C points past the staged entries,
+    whose product row has to come out empty."""
+    g = np.random.default_rng(17)
+    n = 900
+    rp, ci, va = [0], [], []
+    for i in range(n):
+        k = 0 if i % 5 == 4 else 60 if i // 128 % 2 == 0 else 4
+        c = np.unique(np.append(g.integers(0, n, k), i)) if k else np.zeros(0, np.int64)
+        v = np.where(c == i, 1.0, np.where(c % 5 == 4, 1.0, 0.4) * g.uniform(0.5, 1.0, c.size) / max(k, 1))
+        rp.append(rp[-1] + c.size)
+        ci.append(c)
+        va.append(v)
+    rp, ci, va = np.array(rp, np.int32), np.concatenate(ci).astype(np.int32), np.concatenate(va)
+    H = _check(pair, rp, ci, va, distance=distance, nair=nair, theta=0.5, max_levels=3, max_coarse=10)
+    assert H.nlev >= 2
+    staged = 128 * 32   # entries a block holds at this average row length
+    assert rp[-1] * 160 // n > staged
+    L = H.level(0)
+    assert any(rp[i] == rp[i + 1] and rp[i] - rp[i // 128 * 128] > staged for i in L.cpts)
