@@ -1592,7 +1592,8 @@ __global__ void k_rap(int nrows_work, const int *worklist, const int *cpts, cons
             const int key = sl < cap ? keys[sl] : -1;
             const double v = sl < cap ? vals[sl] : 0.0;
             const bool k_ = key >= 0 && !(filt && key != ic && fabs(v) < thr);
-            const unsigned msk = __ballot_sync(FULL, k_) & gmask;   // (every slot of the pass is read)
+            const unsigned msk = __ballot_sync(FULL, k_) & gmask;
+            __syncwarp();   // every slot of the pass is read before one is written (a ballot orders no memory)
             if (k_) {
                 const int off = m + __popc(msk & ((1u << lane) - 1u));
                 keys[off] = key;

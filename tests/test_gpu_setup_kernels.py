@@ -166,3 +166,13 @@ def test_rows_without_entries(pair, distance, nair):
     assert rp[-1] * 160 // n > staged
     L = H.level(0)
     assert any(rp[i] == rp[i + 1] and rp[i] - rp[i // 128 * 128] > staged for i in L.cpts)
+
+
+@pytest.mark.parametrize("entries,n", [(6, 127), (30, 400), (120, 700), (900, 1500)])
+def test_galerkin_tables_packed_with_filter(pair, entries, n):
+    """Rows of every Galerkin table class (shared tables by 8 lanes and by a warp, global
+    tables) with the filter on, so that kept entries move over dropped ones in the table."""
+    rp, ci, va = _matrix(n, lambda i: entries if i % 5 else 3, 40 + entries)
+    H = _check(pair, rp, ci, va, distance=1, theta=0.99, eps_R=0.97, phi_A=0.3, max_levels=2, max_coarse=10)
+    K = O.Hierarchy(rp, ci, va, O.default_params(distance=1, theta=0.99, eps_R=0.97, max_levels=2, max_coarse=10))
+    assert H.level(1).nnz < K.level(1).nnz
