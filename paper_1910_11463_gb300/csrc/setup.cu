@@ -631,7 +631,8 @@ __global__ void __launch_bounds__(128) k_nair(int nc, const int *cpts, const int
         const int e = e0 + g;
         const double z = e < np ? t[e] : 0.0;
         const bool k_ = e < np && !singular && !(phi_R > 0.0 && fabs(z) < thr);
-        const unsigned b = (__ballot_sync(FULL, k_) >> q0) & 0xffu;   // (t of this pass is read)
+        const unsigned b = (__ballot_sync(FULL, k_) >> q0) & 0xffu;
+        __syncwarp();   // t of this pass is read before zval, which may be its place, is written
         if (k_) {
             const int off = base + kept + __popc(b & ((1u << g) - 1u));
             zcol[off] = pat[e];

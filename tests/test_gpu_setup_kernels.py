@@ -176,3 +176,14 @@ def test_galerkin_tables_packed_with_filter(pair, entries, n):
     H = _check(pair, rp, ci, va, distance=1, theta=0.99, eps_R=0.97, phi_A=0.3, max_levels=2, max_coarse=10)
     K = O.Hierarchy(rp, ci, va, O.default_params(distance=1, theta=0.99, eps_R=0.97, max_levels=2, max_coarse=10))
     assert H.level(1).nnz < K.level(1).nnz
+
+
+@pytest.mark.parametrize("phi_R", [0.0, 0.3])
+@pytest.mark.parametrize("entries,n", [(7, 300), (18, 700), (30, 900)])
+def test_nair_pattern_sizes(pair, entries, n, phi_R):
+    """nAIR rows on both sides of the 96 unknowns kept in shared memory, with and without
+    the filter that compacts the others in place."""
+    rp, ci, va = _matrix(n, lambda i: entries if i % 3 else max(1, entries // 4), 80 + entries)
+    _check(pair, rp, ci, va, nair=1, phi_R=phi_R, theta=0.5, max_levels=2, max_coarse=10)
+    z = np.diff(O.Hierarchy(rp, ci, va, O.default_params(nair=1, theta=0.5, max_levels=2, max_coarse=10)).level(0).zrowptr)
+    assert z.min() < 90 and (entries == 7) == (z.max() <= 96)
