@@ -104,7 +104,8 @@ typedef struct {
     int n;              /* rows = columns */
     int nnz;            /* rowptr[n] */
     const int *rowptr;  /* n + 1 */
-    const int *col;     /* nnz, ascending within a row */
+    const int *col;     /* nnz, ascending within a row (a repeated column: products and
+                         * strength take every entry, a lAIR local system the last) */
     const double *val;  /* nnz */
 } pair_csr;
 

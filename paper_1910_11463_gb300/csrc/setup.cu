@@ -547,6 +547,23 @@ __device__ __forceinline__ int pat_find(const int *pat, int np, int k) {
     return -1;
 }
 
+// A caller's matrix may repeat a column within a row (its entries ascend, so the repeats
+// are neighbours).  Products and strength take every entry; a local system takes the last.
+__device__ __forceinline__ bool last_of_run(int p, int p1, const int *col) { return p + 1 >= p1 || col[p + 1] != col[p]; }
+
+// f(p) for the marked entries (S_RF) of the run of one column that holds the marked entry
+// p, in order, by the lane of the first of them (lanes of a group hold neighbouring
+// entries, and only one may touch the column's unknown)
+template <class F>
+__device__ __forceinline__ void marked_run(int p, int p0, int p1, const int *col, const uint8_t *S, F &&f) {
+    const int c = col[p];
+    for (int q = p - 1; q >= p0 && col[q] == c; --q)
+        if (S[q] & S_RF) return;
+    f(p);
+    for (int q = p + 1; q < p1 && col[q] == c; ++q)
+        if (S[q] & S_RF) f(q);
+}
+
 // ---- nAIR of degree 1 (Neumann series cut after the linear term) -----------
 // On the distance-2 pattern (sorted, from k_lair_pattern2):
 //   t_k = a_ik for strong F neighbours k of i (else 0); for every strong F
@@ -555,8 +572,8 @@ __device__ __forceinline__ int pat_find(const int *pat, int np, int k) {
 //   z_k = -(t_k * (1/a_kk)), i.e. Z_i = -A_CF^s[i,:] (I + N) D^{-1} with
 //   N = I - D^{-1} A_FF^s.  A zero diagonal on the way empties the row (counted
 //   as singular).
-// Eight lanes per C row: lanes across a neighbour's row (its columns are distinct, so each
-// t_k still takes its terms in the order of j), pattern and t in shared memory up to
+// Eight lanes per C row: lanes across a neighbour's row (one lane takes all entries of a
+// column, so each t_k takes its terms in the row's order), pattern and t in shared memory up to
 // NAIR_SH unknowns, in the row's slots of cand and zval beyond.  (A thread per row that searched and
 // accumulated in global memory took 1.6 ms a level on 27^3, 8 directions.)
 constexpr int NAIR_SH = 96;
@@ -585,7 +602,8 @@ __global__ void __launch_bounds__(128) k_nair(int nc, const int *cpts, const int
     __syncwarp();
     const int p0 = has ? rowptr[i] : 0, p1 = has ? rowptr[i + 1] : 0;
     for (int p = p0 + g; p < p1; p += 8)
-        if (S[p] & S_RF) t[pat_find(pat, np, col[p])] = val[p];
+        if (S[p] & S_RF)
+            marked_run(p, p0, p1, col, S, [&](int q) { t[pat_find(pat, np, col[q])] = val[q]; });
     __syncwarp();
     bool singular = false;
     int len = p1 - p0;
@@ -606,7 +624,7 @@ __global__ void __launch_bounds__(128) k_nair(int nc, const int *cpts, const int
                 for (int q = s0 + g; q < s1; q += 8) {
                     if (!(S[q] & S_RF)) continue;
                     const int e = pat_find(pat, np, col[q]);
-                    t[e] = fma(a, -(val[q] * r), t[e]);
+                    marked_run(q, s0, s1, col, S, [&](int k) { t[e] = fma(a, -(val[k] * r), t[e]); });
                 }
             __syncwarp();
             m &= m - 1;
@@ -726,7 +744,7 @@ __global__ void k_lair_solve_dense(int nwork, const int *worklist, const int *cp
                 }
             }
             for (int p = rowptr[i] + g; p < rowptr[i + 1]; p += G) {
-                int r = pat_find(pat, np, col[p]);
+                int r = last_of_run(p, rowptr[i + 1], col) ? pat_find(pat, np, col[p]) : -1;
                 if (r >= 0) y[r] = -val[p];
             }
         }
@@ -1051,20 +1069,19 @@ __global__ void k_lair_solve_mask(int nwork, const int *worklist, const int *cpt
             for (int k = 0; k < W; ++k) x.w[k] = 0;
             const int c = g + G * t, j = c < np ? pat[c] : 0, p1 = c < np ? rowptr[j + 1] : 0;
             for (int p = c < np ? rowptr[j] : 0; p < p1; p += 4) {
-                int cc[4], r[4];
+                int cc[5], r[4];
                 double vv[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    cc[u] = p + u < p1 ? col[p + u] : -1;
-                    vv[u] = p + u < p1 ? val[p + u] : 0.0;
-                }
+                for (int u = 0; u < 5; ++u) cc[u] = p + u < p1 ? col[p + u] : -1;
 #pragma unroll
-                for (int u = 0; u < 4; ++u) r[u] = find(cc[u]);
+                for (int u = 0; u < 4; ++u) vv[u] = p + u < p1 ? val[p + u] : 0.0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) r[u] = cc[u] != cc[u + 1] ? find(cc[u]) : -1;   // (see last_of_run)
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
                     if (r[u] >= 0) {
                         M[(size_t)c * ld + r[u]] = vv[u];
-                        x.flip(r[u]);   // (a row holds a column once)
+                        x.flip(r[u]);
                         mxb = max(mxb, absbits(vv[u]));
                     }
             }
@@ -1072,7 +1089,7 @@ __global__ void k_lair_solve_mask(int nwork, const int *worklist, const int *cpt
         }
         if (has)
             for (int p = rowptr[i] + g; p < rowptr[i + 1]; p += G) {
-                const int r = find(col[p]);
+                const int r = last_of_run(p, rowptr[i + 1], col) ? find(col[p]) : -1;
                 if (r >= 0) ys[r] = -val[p];
             }
         __syncwarp();

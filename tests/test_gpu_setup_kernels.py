@@ -187,3 +187,64 @@ def test_nair_pattern_sizes(pair, entries, n, phi_R):
     _check(pair, rp, ci, va, nair=1, phi_R=phi_R, theta=0.5, max_levels=2, max_coarse=10)
     z = np.diff(O.Hierarchy(rp, ci, va, O.default_params(nair=1, theta=0.5, max_levels=2, max_coarse=10)).level(0).zrowptr)
     assert z.min() < 90 and (entries == 7) == (z.max() <= 96)
+
+
+def _level0(pair, rp, ci, va, **kw):
+    G = pair.Hierarchy([tuple(torch.as_tensor(a, device="cuda") for a in (rp, ci, va))],
+                       pair.default_air_params(precision=0, **kw))
+    return G.level(0, 0)
+
+
+@pytest.mark.parametrize("entries,distance", [(6, 1), (22, 1), (55, 1), (120, 1), (8, 2)])
+def test_repeated_columns_local_solves(pair, entries, distance):
+    """Entries repeated in front of the stored ones, weaker than eps_R: the strength and the
+    patterns stay as they are, and the local systems take the last value of a column."""
+    n = 500
+    rp, ci, va = _coupled(n, entries, 90 + entries)
+    g = np.random.default_rng(entries)
+    rows = np.repeat(np.arange(n), np.diff(rp))
+    again = 1 + (g.random(ci.size) < 0.4) + (g.random(ci.size) < 0.1)   # one to three times
+    first = np.zeros(again.sum(), bool)
+    first[np.cumsum(again) - 1] = True   # the last of a run is the stored entry
+    vd = np.where(first, np.repeat(va, again), 1e-5 * g.uniform(-1.0, 1.0, first.size))
+    rd = np.concatenate([[0], np.cumsum(np.bincount(rows, weights=again, minlength=n))]).astype(np.int32)
+    kw = dict(distance=distance, theta=0.6, max_levels=2, max_coarse=10)
+    a = _level0(pair, rd, np.repeat(ci, again).astype(np.int32), vd, **kw)
+    b = O.Hierarchy(rp, ci, va, O.default_params(**kw)).level(0)
+    assert np.array_equal(a.cf, b.cf) and np.array_equal(a.zrowptr, b.zrowptr) and np.array_equal(a.zcol, b.zcol)
+    assert np.array_equal(a.zval.view(np.uint64), b.zval.view(np.uint64))
+
+
+@pytest.mark.parametrize("entries", [4, 20])
+def test_repeated_columns_nair(pair, entries):
+    """Every off-diagonal entry stored as two halves, all of them strong: each term of the
+    Neumann sum counts, in order.  A t_k of m terms is off by at most (m + 2) roundings of
+    the sum of their magnitudes."""
+    n = 400
+    rp, ci, va = _matrix(n, lambda i: entries, 70 + entries)
+    rows = np.repeat(np.arange(n), np.diff(rp))
+    twice = np.where(rows == ci, 1, 2)
+    rd = np.concatenate([[0], np.cumsum(np.bincount(rows, weights=twice, minlength=n))]).astype(np.int32)
+    cd, vd = np.repeat(ci, twice).astype(np.int32), np.repeat(va / twice, twice)
+    L = _level0(pair, rd, cd, vd, nair=1, theta=0.5, eps_R=0.01, max_levels=2, max_coarse=10)
+    diag = va[rows == ci]
+    strong = []   # (column, value) of each row's strong F entries, in order
+    for i in range(n):
+        c, v = cd[rd[i]:rd[i + 1]], vd[rd[i]:rd[i + 1]]
+        o = c != i
+        m = np.abs(v[o]).max() if o.any() else 0.0
+        keep = o & (np.abs(v) >= 0.01 * m) & (L.cf[c] == 0)
+        strong.append(list(zip(c[keep], v[keep])))
+    assert len(L.cpts) > 20
+    for r, i in enumerate(L.cpts):
+        t = {k: v for k, v in strong[i]}   # (the last of a repeated column)
+        mag = {k: abs(v) for k, v in t.items()}
+        for j, a in strong[i]:
+            for k, v in strong[j]:
+                t[k] = t.get(k, 0.0) - a * v / diag[j]
+                mag[k] = mag.get(k, 0.0) + abs(a * v / diag[j])
+        s, e = L.zrowptr[r], L.zrowptr[r + 1]
+        assert list(L.zcol[s:e]) == sorted(t)
+        terms = 2 + 4 * len(strong[i])
+        for k, z in zip(L.zcol[s:e], L.zval[s:e]):
+            assert abs(z + t[k] / diag[k]) <= (terms + 2) * 4.5e-16 * mag[k] / abs(diag[k]), (i, k)
