@@ -1061,6 +1061,9 @@ __global__ void k_coarsest(const int *seg_row0, const int *seg_n, const int *seg
                     sweeps, cs_sm, &cs_bad);
 }
 
+__device__ __forceinline__ bool zero_weight(float w) { return w == 0.0f; }
+__device__ __forceinline__ bool zero_weight(double w) { return (__double_as_longlong(w) << 1) == 0; }   // (not on the FP64 pipe)
+
 // ---- coarsest level: the sweeps as one dense product ----------------------------------
 // The coarse_sweeps Jacobi sweeps from zero are linear in b: x = B b with
 // B = sum_{k < sweeps} (I - D^{-1} A)^k D^{-1}, an nr x nr matrix of a segment of nr rows.
@@ -1090,8 +1093,8 @@ __global__ void __launch_bounds__(4 * CD_ROWS) k_coarsest_dense(const int *seg_r
     __syncthreads();
     T acc = T(0);
 #pragma unroll
-    for (int i = 0; i < NI; ++i)
-        if (i < ni) acc += w[i] * sb[4 * i + q];
+    for (int i = 0; i < NI; ++i)   // (a zero weight adds nothing, also to rows an infinity or NaN in b does not reach)
+        if (i < ni && !zero_weight(w[i])) acc += w[i] * sb[4 * i + q];
     acc += __shfl_xor_sync(0xffffffffu, acc, 1);
     acc += __shfl_xor_sync(0xffffffffu, acc, 2);
     const int r = blockIdx.y * CD_ROWS + (t >> 2);

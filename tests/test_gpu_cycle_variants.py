@@ -92,3 +92,27 @@ def test_first_sweep_through_p_columns(pair, n, far, f_sweeps):
     assert H.nlev >= 2
     xo = H.vcycle(b, x0.copy())
     assert np.linalg.norm(x - xo) <= 1e-12 * np.linalg.norm(xo)
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+@pytest.mark.parametrize("precision,n", [(0, 33), (0, 100), (1, 100)])
+def test_nonfinite_right_hand_side_reaches_the_rows_the_sweeps_reach(pair, precision, n, bad):
+    """One infinity or NaN in the right-hand side of a coarsest level: the rows that the
+    sweeps couple to it, and no others, are not finite afterwards."""
+    from oracle import oracle as O
+    g = np.random.default_rng(n)
+    A = np.eye(n) + np.tril(g.uniform(-0.5, 0.5, (n, n)) * (g.random((n, n)) < 0.05), -1)
+    ci = [np.nonzero(r)[0] for r in A]
+    rp = np.concatenate([[0], np.cumsum([len(c) for c in ci])]).astype(np.int32)
+    col = np.concatenate(ci).astype(np.int32)
+    val = np.concatenate([A[i, c] for i, c in enumerate(ci)])
+    b = g.uniform(1.0, 2.0, n)
+    b[n // 4] = bad
+    kw = dict(max_coarse=1000, coarse_sweeps=4)
+    h = pair.Hierarchy([tuple(torch.as_tensor(a, device="cuda") for a in (rp, col, val))],
+                       pair.default_air_params(precision=precision, **kw))
+    x = h.vcycle(torch.as_tensor(b, device="cuda"), torch.zeros(n, dtype=torch.float64, device="cuda")).cpu().numpy()
+    xo = O.Hierarchy(rp, col, val, O.default_params(**kw)).vcycle(b, np.zeros(n))
+    ok = np.isfinite(xo)
+    assert 0 < ok.sum() < n and np.array_equal(np.isfinite(x), ok)
+    assert np.allclose(x[ok], xo[ok], rtol=1e-12 if precision == 0 else 2e-5, atol=0)   # (condition below 13)
