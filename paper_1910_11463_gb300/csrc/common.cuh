@@ -206,8 +206,11 @@ constexpr int SD_MAXE = 8;
 // memory; a level with a larger one gets a SELL copy of its coarsest rows instead.
 constexpr int CS_SMEM = 40 * 1024;
 // Coarsest segments of at most CD_MAX rows (the library's max_coarse is 100) apply their
-// sweeps as one dense product, CD_ROWS rows to a block.
+// sweeps as one dense product, CD_ROWS rows to a block, while the products of all matrices
+// of the level fit CD_BYTES (2600 matrices of 100 rows in FP64; larger batches sweep in
+// place, with no memory beyond the operator's).
 constexpr int CD_MAX = 128, CD_ROWS = 32;
+constexpr size_t CD_BYTES = 256u << 20;
 struct SweepPlan {
     int nb = 0, nlev = 0, ncomp = 0;
     int *list = nullptr;                     // single elements, level by level

@@ -1073,7 +1073,8 @@ __device__ __forceinline__ bool zero_weight(double w) { return (__double_as_long
 // sweeping the unit vectors) and kept in the cycle precision; its product reads it before
 // the wait for the restriction, so 4 lanes a row are left with nr / 4 multiply-adds.  8^3
 // S2 in FP64 26.7 -> 20.7 ms, 13^3 S4 50.5 -> 48.0, 7^3 tet FP64 gradient 131 -> 105.
-// Segments past CD_MAX rows keep the sweeps (B grows with nr^2).
+// Segments past CD_MAX rows keep the sweeps (B grows with nr^2), and so does a level whose
+// products together would take more than CD_BYTES.
 template <class T>
 __global__ void __launch_bounds__(4 * CD_ROWS) k_coarsest_dense(const int *seg_row0, const int *seg_n, const int *off,
                                                                 const T *B, const T *b, T *x, const int *any) {
@@ -1433,9 +1434,16 @@ void coarsest_dense(Hier &h, Level &L) {
             at += (long long)((nr + CD_ROWS - 1) / CD_ROWS) * 4 * ((nr + 3) / 4);
         }
     const size_t es = h.prm.precision >= 1 ? sizeof(float) : sizeof(double);
+    const size_t bytes = (size_t)at * CD_ROWS * es;
+    if (bytes > CD_BYTES) return;
+    try {
+        L.cB = dmalloc<char>(bytes, s);
+    } catch (const Error &e) {
+        if (e.st != PAIR_ERR_OOM) throw;
+        return;   // no room for it: the sweeps need nothing more than is there
+    }
     L.cseg_max = mx;
-    L.cB = dmalloc<char>((size_t)at * CD_ROWS * es, s);
-    PR_CUDA(cudaMemsetAsync(L.cB, 0, (size_t)at * CD_ROWS * es, s));   // the columns past nr of a row's last four
+    PR_CUDA(cudaMemsetAsync(L.cB, 0, bytes, s));   // the columns past nr of a row's last four
     L.d_cB_off = dmalloc<int>(off.size(), s);
     PR_CUDA(cudaMemcpyAsync(L.d_cB_off, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice, s));
     const dim3 grid(L.n_cseg, (mx + CD_COLS - 1) / CD_COLS);

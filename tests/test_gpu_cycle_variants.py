@@ -116,3 +116,40 @@ def test_nonfinite_right_hand_side_reaches_the_rows_the_sweeps_reach(pair, preci
     ok = np.isfinite(xo)
     assert 0 < ok.sum() < n and np.array_equal(np.isfinite(x), ok)
     assert np.allclose(x[ok], xo[ok], rtol=1e-12 if precision == 0 else 2e-5, atol=0)   # (condition below 13)
+
+
+_MANY = """
+import numpy as np, torch
+from paper_1910_11463_gb300 import pair
+count, n, sweeps = 6000, 100, 3
+g = np.random.default_rng(0)
+rp = np.concatenate([[0], 1 + 2 * np.arange(n)]).astype(np.int32)
+col = np.concatenate([[0]] + [[i - 1, i] for i in range(1, n)]).astype(np.int32)
+val = np.concatenate([[1.0]] + [[g.uniform(-0.5, 0.5), 1.0] for i in range(1, n)])
+dev = tuple(torch.as_tensor(a, device="cuda") for a in (rp, col, val))
+prm = pair.default_air_params(precision=0, coarse_sweeps=sweeps)
+b = torch.as_tensor(np.tile(g.standard_normal(n), count), device="cuda")
+x = torch.zeros_like(b)
+small = pair.Hierarchy([dev] * 2, prm).vcycle(b[:2 * n].clone(), torch.zeros(2 * n, dtype=torch.float64, device="cuda"))
+torch.cuda.synchronize()
+free = torch.cuda.mem_get_info()[0]
+h = pair.Hierarchy([dev] * count, prm)
+h.vcycle(b, x)
+torch.cuda.synchronize()
+print((free - torch.cuda.mem_get_info()[0]) / 2 ** 20)
+x = x.view(count, n)
+assert torch.equal(x, x[:1].expand(count, n))
+assert torch.allclose(x[0], small[:n], rtol=1e-13, atol=1e-13)
+"""
+
+
+def test_coarsest_products_are_bounded_in_memory(pair):
+    """6000 matrices of 100 rows: their products would take 590 MB, the operators, vectors
+    and the setup's scratch take less than 200."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _MANY], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert float(r.stdout.split()[-1]) < 400.0
