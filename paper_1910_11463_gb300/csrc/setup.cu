@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(256) k_lair_pattern2_big(const int *big, const
 // unknowns, with shared workspaces sized to the bin (the smaller they are, the more
 // systems are in flight per SM); global workspaces beyond 64, and a dense kernel past 256
 constexpr int LAIR_CLASSES = 12;
-constexpr int LAIR_BIG = LAIR_CLASSES - 1;
+constexpr int LAIR_BIG = LAIR_CLASSES - 1, LAIR_SLOT = LAIR_BIG - 2;   // dense; first class with global slots
 __device__ __forceinline__ int lair_class(int np) {
     return np <= 4 ? 0 : np <= 6 ? 1 : np <= 8 ? 2 : np <= 12 ? 3 : np <= 16 ? 4 : np <= 24 ? 5 : np <= 32 ? 6
          : np <= 48 ? 7 : np <= 64 ? 8 : np <= 128 ? 9 : np <= 256 ? 10 : 11;
@@ -1679,9 +1679,15 @@ __global__ void k_big_rows(int nbig, const int *list, const int *npat, long long
 }
 
 
-__global__ void k_lair_classes(int nc, const int *npat, int8_t *cls) {
+// class of every system, and the largest system of each class with global slots (bmax)
+__global__ void k_lair_classes(int nc, const int *npat, int8_t *cls, int *bmax) {
     int ic = blockIdx.x * blockDim.x + threadIdx.x;
-    if (ic < nc) cls[ic] = (int8_t)lair_class(npat[ic]);
+    const int np = ic < nc ? npat[ic] : 0, c = lair_class(np);
+    if (ic < nc) cls[ic] = (int8_t)c;
+    for (int k = LAIR_SLOT; k < LAIR_BIG; ++k) {
+        const int mx = __reduce_max_sync(0xffffffffu, c == k ? np : 0);
+        if (mx > 0 && (threadIdx.x & 31) == 0) atomicMax(&bmax[k - LAIR_SLOT], mx);
+    }
 }
 
 __global__ void k_rap_classes(int nc, const int *U, int8_t *cls) {
@@ -2301,13 +2307,17 @@ void build_hierarchy(Hier &h) {
         } else {
             // rows binned by system size; shared memory per warp sized to the bin
             int8_t *ccls = dmalloc<int8_t>(nc, s);
-            k_lair_classes<<<blocks_for(nc, BS), BS, 0, s>>>(nc, npat, ccls);
+            int *dbmax = dmalloc<int>(LAIR_BIG - LAIR_SLOT, s);
+            PR_CUDA(cudaMemsetAsync(dbmax, 0, sizeof(int) * (LAIR_BIG - LAIR_SLOT), s));
+            k_lair_classes<<<blocks_for(nc, BS), BS, 0, s>>>(nc, npat, ccls, dbmax);
             PR_LAUNCH();
             int hc[LAIR_CLASSES], hstart[LAIR_CLASSES];
             int *list = dmalloc<int>(nc, s);
             partition_by_class(ccls, nc, LAIR_CLASSES, list, hstart, hc, s);
             dfree(ccls, s);
-            const int cls_n[LAIR_CLASSES] = {4, 6, 8, 12, 16, 24, 32, 48, 64, 128, 256, 0};
+            int cls_n[LAIR_CLASSES] = {4, 6, 8, 12, 16, 24, 32, 48, 64, 0, 0, 0};
+            if (hc[LAIR_SLOT] || hc[LAIR_SLOT + 1]) d2h(cls_n + LAIR_SLOT, dbmax, LAIR_BIG - LAIR_SLOT, s);
+            dfree(dbmax, s);
             // blocks of one to four warps, so that the shared memory of an SM fills evenly
             auto mask_bin = [&](int c, auto kern, int G, int R) {
                 if (!hc[c]) return;
@@ -2322,6 +2332,7 @@ void build_hierarchy(Hier &h) {
                 PR_LAUNCH();
             };
             // more than 64 unknowns: a warp a system, its workspace a slot of global memory
+            // for the largest system of the class
             auto mask_big = [&](int c, auto kern, int R, unsigned warps) {
                 if (!hc[c]) return;
                 const int nm = cls_n[c];
@@ -2337,8 +2348,8 @@ void build_hierarchy(Hier &h) {
             for (int c = 3; c <= 4; ++c) mask_bin(c, k_lair_solve_mask<8, 2, false>, 8, 2);
             for (int c = 5; c <= 6; ++c) mask_bin(c, k_lair_solve_mask<16, 2, false>, 16, 2);
             for (int c = 7; c <= 8; ++c) mask_bin(c, k_lair_solve_mask<32, 2, false>, 32, 2);
-            mask_big(9, k_lair_solve_mask<32, 4, true>, 4, 152u * 20u);
-            mask_big(10, k_lair_solve_mask<32, 8, true>, 8, 152u * 12u);
+            mask_big(LAIR_SLOT, k_lair_solve_mask<32, 4, true>, 4, 152u * 20u);
+            mask_big(LAIR_SLOT + 1, k_lair_solve_mask<32, 8, true>, 8, 152u * 12u);
             int nbig = hc[LAIR_BIG];
             if (nbig > 0) {
                 long long *goff = dmalloc<long long>(nbig + 1, s);

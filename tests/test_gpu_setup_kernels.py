@@ -248,3 +248,51 @@ def test_repeated_columns_nair(pair, entries):
         terms = 2 + 4 * len(strong[i])
         for k, z in zip(L.zcol[s:e], L.zval[s:e]):
             assert abs(z + t[k] / diag[k]) <= (terms + 2) * 4.5e-16 * mag[k] / abs(diag[k]), (i, k)
+
+
+def _wide(n, k, seed):
+    """Even rows couple most strongly to one even row and, weaker, to k odd ones; odd rows
+    couple to one even row.  With theta = 1 the C rows are even, and their local systems
+    have about k unknowns."""
+    g = np.random.default_rng(seed)
+    rp, ci, va = [0], [], []
+    for i in range(n):
+        e = 2 * int(g.integers(0, n // 2 - 1))
+        e += 2 * (e >= i)   # an even row other than i
+        odd = np.zeros(0, np.int64) if i % 2 else 1 + 2 * g.choice(n // 2, k, replace=False)
+        c = np.sort(np.concatenate([[i, e], odd]))
+        va.append(np.where(c == i, 2.0, np.where(c == e, 0.5, 0.25 * g.uniform(0.5, 1.0, c.size) / k ** 0.5)))
+        ci.append(c)
+        rp.append(rp[-1] + c.size)
+    return np.array(rp, np.int32), np.concatenate(ci).astype(np.int32), np.concatenate(va)
+
+
+_SLOTS = """
+import torch
+import tests.test_gpu_setup_kernels as T
+from paper_1910_11463_gb300 import pair
+kw = dict(theta=1.0, eps_R=0.01, max_levels=2, max_coarse=10, precision=0)
+cuda = lambda m: [tuple(torch.as_tensor(a, device="cuda") for a in m)]
+pair.Hierarchy(cuda(T._wide(600, 130, 1)), pair.default_air_params(**kw))
+m = cuda(T._wide(16000, 130, 2))
+torch.cuda.synchronize()
+free = torch.cuda.mem_get_info()[0]
+h = pair.Hierarchy(m, pair.default_air_params(**kw))
+torch.cuda.synchronize()
+print((free - torch.cuda.mem_get_info()[0]) / 2 ** 20)
+"""
+
+
+def test_workspaces_of_large_local_systems(pair):
+    """Thousands of systems of about 130 unknowns take slots of their size (250 MB for the
+    1824 resident warps), not of the class's largest (960 MB); bits as in the oracle."""
+    import os
+    import subprocess
+    import sys
+    H = _check(pair, *_wide(600, 130, 1), theta=1.0, eps_R=0.01, max_levels=2, max_coarse=10)
+    z = np.diff(H.level(0).zrowptr)
+    assert 128 < np.median(z) < 140
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _SLOTS], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert float(r.stdout.split()[-1]) < 600.0
