@@ -1559,6 +1559,18 @@ __global__ void k_level_counts_dir(int n, const int *rowptr, const int8_t *cf, c
             if (c[k]) atomicAdd(&out[4LL * d + k], c[k]);
     }
 }
+// column index of an entry: 4 bytes, or 2 in a store with 16-bit offsets
+double col_bytes(const Sell &S) { return S.col16 ? 2.0 : 4.0; }
+// The F sweeps of a level relaxed from SELL copies: each reads, per F row, its split
+// position (row index and entry offset), b, dinv and its input value, writes its output
+// value, and reads its entries (column + value).  The first one reads P columns instead,
+// also the row's own, and moves the C rows' coarse values: per C row its index and the
+// value, written to both buffers.  Gathered neighbour values are taken as cached (the
+// vector is far smaller than L2).
+double sell_f_bytes(const Hier &h, const Level &L, double nF, double nC, double eF, double sT) {
+    const double first = nF * (12 + 4 * sT) + eF * ((L.sF.pcol16 ? 2.0 : 4.0) + sT) + nC * (4 + 3 * sT);
+    return first + (h.prm.f_sweeps - 1) * (nF * (8 + 4 * sT) + eF * (col_bytes(L.sF) + sT));
+}
 }  // namespace
 
 void level0_bytes(Hier &h) {
@@ -1577,8 +1589,7 @@ void level0_bytes(Hier &h) {
         for (size_t l = 0; l + 1 < h.lev.size(); ++l) {
             const Level &L = h.lev[l];
             if (L.nc <= 0) continue;
-            const double cb = L.sZ.col16 ? 2.0 : 4.0;
-            h.bytes_xfer += (double)L.nc * (12 + 2 * sT) + (double)L.nnzZ * (cb + sT);
+            h.bytes_xfer += (double)L.nc * (12 + 2 * sT) + (double)L.nnzZ * (col_bytes(L.sZ) + sT);
             // (SELL levels: the C rows' scatter, by the first F sweep)
             if (l == 0 && h.bsr0) h.bytes_xfer += (double)(L.nF + L.nC) * (5 + sT) + (double)L.nC * sT;
         }
@@ -1588,10 +1599,8 @@ void level0_bytes(Hier &h) {
     const double xfold = h.inner ? 8.0 : 16.0;
     cudaStream_t s = h.stream;
     {
-        // coarse levels: each F sweep reads, per F row, its split position (row index and
-        // entry offset), b, dinv and its input value, writes its output value, and reads
-        // its entries (column + value); the C sweep likewise over the C rows.  Gathered
-        // neighbour values are taken as cached (the vector is far smaller than L2).
+        // coarse levels: the F sweeps (sell_f_bytes); the C sweep likewise over the C rows;
+        // the last F sweep writes its rows a second time
         double sT = h.prm.precision >= 1 ? 4.0 : 8.0;
         unsigned long long *cnt = dmalloc<unsigned long long>(4, s);
         for (size_t l = 1; l + 1 < h.lev.size(); ++l) {
@@ -1603,11 +1612,8 @@ void level0_bytes(Hier &h) {
             unsigned long long c[4];
             PR_CUDA(cudaMemcpyAsync(c, cnt, sizeof c, cudaMemcpyDeviceToHost, s));
             PR_CUDA(cudaStreamSynchronize(s));
-            // column index: 4 bytes, or 2 in a store with 16-bit offsets
-            const double cbF = L.sF.col16 ? 2.0 : 4.0, cbC = L.sC.col16 ? 2.0 : 4.0;
-            double fpass = (double)c[0] * (8 + 4 * sT) + (double)c[2] * (cbF + sT);
-            double cpass = (double)c[1] * (8 + 4 * sT) + (double)c[3] * (cbC + sT);
-            h.bytes_relaxc += h.prm.f_sweeps * fpass + cpass + (double)c[1] * (4 + 3 * sT) + (double)c[0] * sT;
+            h.bytes_relaxc += sell_f_bytes(h, L, (double)c[0], (double)c[1], (double)c[2], sT) + (double)c[0] * sT +
+                              (double)c[1] * (8 + 4 * sT) + (double)c[3] * (col_bytes(L.sC) + sT);
         }
         dfree(cnt, s);
         // grid-wide coarsest sweeps: the first reads each row's split position, b and
@@ -1618,14 +1624,15 @@ void level0_bytes(Hier &h) {
             double nz = 0;
             for (int d = 0; d < h.ndir; ++d)
                 if (L.nrows[d] > 0 && L.coarsest[d]) nz += L.nnzdir[d];
-            const double nx = L.sX.nrows, cb = L.sX.col16 ? 2.0 : 4.0;
+            const double nx = L.sX.nrows, cb = col_bytes(L.sX);
             h.bytes_relaxc += nx * (4 + 3 * sT) + (h.prm.coarse_sweeps - 1) * (nx * (8 + 4 * sT) + nz * (cb + sT));
         }
     }
     if (!h.bsr0) {
         // CSR level 0 (tetrahedra): residual reads every entry (column + FP64 value), b
-        // and x, writes r; the relaxation counts as on coarse levels, except that the
-        // last F sweep and the C sweep add into x64 (read + write) instead of writing
+        // and x, writes r; the relaxation counts as on coarse levels, except that the last F
+        // sweep adds its rows into x64 (read + write) instead of writing them a second time,
+        // and the C sweep instead of writing
         Level &L = h.lev[0];
         double sT = h.prm.precision >= 1 ? 4.0 : 8.0;
         unsigned long long *cnt = dmalloc<unsigned long long>(4 * h.ndir, s);
@@ -1641,9 +1648,8 @@ void level0_bytes(Hier &h) {
                    eC = (double)c[4 * m + 3];
             // outer residual: entries, b and x read, r written (and its r32 copy)
             h.bytes_res0[m] = (eF + eC) * 12 + (nF + nC) * (16 + sT + (h.inner ? 4 : 0));
-            double fpass = nF * (8 + 4 * sT) + eF * (4 + sT);
-            double cpass = nC * (8 + 3 * sT + xfold) + eC * (4 + sT);
-            h.bytes_relax0[m] = h.prm.f_sweeps * fpass + nF * xfold + cpass;
+            h.bytes_relax0[m] = sell_f_bytes(h, L, nF, nC, eF, sT) + nF * xfold + nC * (8 + 3 * sT + xfold) +
+                                eC * (col_bytes(L.sC) + sT);
             // inner residual: row pointer, entries (column + FP32 value), r32 and d read, r written
             if (h.inner) h.bytes_res32[m] = (eF + eC) * 8 + (nF + nC) * 16;
         }

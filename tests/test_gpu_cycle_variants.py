@@ -153,3 +153,51 @@ def test_coarsest_products_are_bounded_in_memory(pair):
     r = subprocess.run([sys.executable, "-c", _MANY], cwd=root, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
     assert float(r.stdout.split()[-1]) < 400.0
+
+
+# the traffic counters of the SELL levels, from the exported hierarchies: 16-bit columns
+# everywhere (n = 5), and a level 0 whose columns take 32 bits and P columns 16 (n = 38)
+@pytest.mark.parametrize("n,f_sweeps", [(5, 1), (5, 3), (38, 2)])
+def test_relaxation_traffic_counters(pair, n, f_sweeps):
+    prob = I.small_tet(n, order=2, seed=4)
+    air = pair.default_air_params(precision=0, theta=0.5, f_sweeps=f_sweeps, max_levels=3, max_coarse=20, coarse_sweeps=1)
+    si = pair.default_si_params(max_iters=1, fixed_iters=1, inner_cycles=1, concurrent=1, timing=1)
+    _, _, info = pair.si_solve_problem(prob, air=air, si=si)
+    assert info["batches"] == 1 and info["n_relax0"] == 1
+    mesh = pair.TetMesh(prob.verts, prob.tets, prob.nbr)
+    st = torch.as_tensor(prob.sigma_t, device="cuda")
+    levels = [[], []]   # per level and direction: rows, entries and widths
+    nx, big = 0, False   # rows of the coarsest level; a segment of it past 40 KB: grid-wide sweeps
+    for m in range(prob.M):
+        h = pair.Hierarchy([pair.dg_assemble_tet(mesh, prob.omega[m], st)], air)
+        assert h.nlevels() == 3
+        X = h.level(0, 2)
+        nx += X.n
+        big |= X.nnz * 12 + X.n * 32 + (X.n + 1) * 4 > 40 * 1024
+        for l in (0, 1):
+            L = h.level(0, l)
+            F = L.cf == 0
+            lens = np.diff(L.rowptr)
+            rows = np.repeat(np.arange(L.n), lens)
+            near = np.abs(L.col - rows) <= 32767
+            pc, fe = L.pmap[L.col], F[rows]
+            org = L.pmap.copy()   # a row's origin: its own P column, else its first entry's
+            p = np.nonzero(fe & (pc >= 0) & (org[rows] < 0))[0][::-1]
+            org[rows[p]] = pc[p]   # (of repeated rows the last assignment, the first entry, stays)
+            pnear = (pc < 0) | (np.abs(pc - org[rows]) <= 32767)
+            levels[l].append((F.sum(), (~F).sum(), lens[F].sum(), lens[~F].sum(), near[fe].all(), near[~fe].all(),
+                              pnear[fe].all()))
+    want = []
+    for l in (0, 1):
+        a = np.array(levels[l], dtype=np.int64)
+        nF, nC, eF, eC = a[:, :4].sum(0)
+        cF, cC, cP = (2 if ok else 4 for ok in a[:, 4:].all(0))
+        if n == 38 and l == 0:
+            assert (cF, cP) == (4, 2)
+        b = nF * (12 + 32) + eF * (cP + 8) + nC * (4 + 24) + (f_sweeps - 1) * (nF * (8 + 32) + eF * (cF + 8))
+        b += (nF * 16 + nC * (8 + 24 + 16) if l == 0 else nF * 8 + nC * (8 + 32)) + eC * (cC + 8)
+        want.append(b)
+    if big:
+        want[1] += nx * (4 + 24)   # the one coarsest sweep: position, b and dinv read, value written
+    for got, w in zip((info["gb_relax0"], info["gb_relaxc"]), want):
+        assert abs(got * 1e9 - w) <= 1e-9 * w
