@@ -296,3 +296,28 @@ def test_workspaces_of_large_local_systems(pair):
     r = subprocess.run([sys.executable, "-c", _SLOTS], cwd=root, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
     assert float(r.stdout.split()[-1]) < 600.0
+
+
+@pytest.mark.parametrize("phi_R", [0.0, 0.1])
+@pytest.mark.parametrize("entries,n,lo,hi", [(110, 600, 65, 128), (160, 700, 65, 256), (240, 900, 129, 256),
+                                             (300, 1000, 129, 400), (420, 1300, 257, 400)])
+def test_lair_solver_bins_past_64(pair, entries, n, lo, hi, phi_R):
+    """Systems of 65-128, 129-256 and more than 256 unknowns that exchange rows (across the
+    words of the row masks) and fill in; some hold two equal rows and are singular."""
+    rp, ci, va = _coupled(n, entries, 60 + entries)
+    for i in range(n // 8, n, n // 4):   # pairs of equal rows
+        s, e = rp[i], rp[i + 1]
+        ci = np.concatenate([ci[:e], ci[s:e], ci[rp[i + 2]:]])
+        va = np.concatenate([va[:e], va[s:e], va[rp[i + 2]:]])
+        rp = np.concatenate([rp[:i + 2], rp[i + 2:] + (2 * e - s - rp[i + 2])]).astype(np.int32)
+    kw = dict(distance=1, theta=0.6, max_levels=2, max_coarse=10)
+    H = _check(pair, rp, ci, va, phi_R=phi_R, **kw)
+    # a singular system's Z row is empty; the others hold their whole pattern without the filter
+    L = O.Hierarchy(rp, ci, va, O.default_params(**kw)).level(0)
+    z = np.diff(L.zrowptr)
+    assert 0 < L.n_singular < len(z) and H.level(0).n_singular == L.n_singular
+    z = z[z > 0]
+    assert z.min() >= lo and z.max() <= hi
+    if (lo, hi) in ((65, 256), (129, 400)):
+        mid = {256: 128, 400: 256}[hi]
+        assert (z <= mid).any() and (z > mid).any()
