@@ -201,3 +201,29 @@ def test_relaxation_traffic_counters(pair, n, f_sweeps):
         want[1] += nx * (4 + 24)   # the one coarsest sweep: position, b and dinv read, value written
     for got, w in zip((info["gb_relax0"], info["gb_relaxc"]), want):
         assert abs(got * 1e9 - w) <= 1e-9 * w
+
+
+# the same in FP32 cycles: the first sweep's gathers, C rows and second target with 16-bit
+# and 32-bit P columns; a cycle's values pass through about 40 roundings of sums of at most
+# a few dozen terms, 6e-8 each against values of the size of x
+@pytest.mark.parametrize("n,far,f_sweeps", [(300, False, 1), (3000, False, 2), (3000, False, 3), (150_000, True, 2)])
+def test_first_sweep_through_p_columns_fp32(pair, n, far, f_sweeps):
+    from oracle import oracle as O
+    g = np.random.default_rng(n + f_sweeps)
+    k = 3
+    off = g.integers(0, n, (n, k)) if far else np.clip(np.arange(n)[:, None] + g.integers(-20, 21, (n, k)), 0, n - 1)
+    off[::9] = np.arange(n)[::9, None]   # rows that depend on nothing
+    r, c = np.repeat(np.arange(n), k), off.ravel()
+    key = np.unique(np.concatenate([r.astype(np.int64) * n + c, np.arange(n, dtype=np.int64) * (n + 1)]))
+    r, c = key // n, (key % n).astype(np.int32)
+    v = np.where(r == c, 1.0, g.uniform(-0.3, 0.3, key.size))
+    rp = np.concatenate([[0], np.cumsum(np.bincount(r, minlength=n))]).astype(np.int32)
+    kw = dict(theta=0.5, max_coarse=50, max_levels=4, f_sweeps=f_sweeps)
+    b, x0 = g.random(n), g.random(n)
+    h = pair.Hierarchy([tuple(torch.as_tensor(a, device="cuda") for a in (rp, c, v))],
+                       pair.default_air_params(precision=1, **kw))
+    x = h.vcycle(torch.as_tensor(b, device="cuda"), torch.as_tensor(x0, device="cuda").clone()).cpu().numpy()
+    H = O.Hierarchy(rp, c, v, O.default_params(**kw))
+    assert H.nlev >= 2
+    xo = H.vcycle(b, x0.copy())
+    assert np.linalg.norm(x - xo) <= 40 * 6e-8 * np.linalg.norm(xo)
