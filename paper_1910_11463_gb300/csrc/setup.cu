@@ -744,8 +744,8 @@ __global__ void k_lair_solve_dense(int nwork, const int *worklist, const int *cp
                 }
             }
             for (int p = rowptr[i] + g; p < rowptr[i + 1]; p += G) {
-                int r = last_of_run(p, rowptr[i + 1], col) ? pat_find(pat, np, col[p]) : -1;
-                if (r >= 0) y[r] = -val[p];
+                int r = pat_find(pat, np, col[p]);
+                if (r >= 0 && last_of_run(p, rowptr[i + 1], col)) y[r] = -val[p];
             }
         }
         __syncwarp();
@@ -971,6 +971,11 @@ struct RowMask {
             if ((r >> 6) == k) b = (w[k] >> (r & 63)) & 1ULL;
         return b;
     }
+    __device__ __forceinline__ void set(int r) {
+#pragma unroll
+        for (int k = 0; k < W; ++k)
+            if (W == 1 || (r >> 6) == k) w[k] |= 1ULL << (r & 63);
+    }
     __device__ __forceinline__ void flip(int r) {
 #pragma unroll
         for (int k = 0; k < W; ++k)
@@ -1068,29 +1073,43 @@ __global__ void k_lair_solve_mask(int nwork, const int *worklist, const int *cpt
 #pragma unroll
             for (int k = 0; k < W; ++k) x.w[k] = 0;
             const int c = g + G * t, j = c < np ? pat[c] : 0, p1 = c < np ? rowptr[j + 1] : 0;
+            int last = -1;
+            bool repeats = false;
+            long long cmax = 0;
             for (int p = c < np ? rowptr[j] : 0; p < p1; p += 4) {
-                int cc[5], r[4];
+                int cc[4], r[4];
                 double vv[4];
 #pragma unroll
-                for (int u = 0; u < 5; ++u) cc[u] = p + u < p1 ? col[p + u] : -1;
+                for (int u = 0; u < 4; ++u) {
+                    cc[u] = p + u < p1 ? col[p + u] : -1;
+                    vv[u] = p + u < p1 ? val[p + u] : 0.0;
+                }
 #pragma unroll
-                for (int u = 0; u < 4; ++u) vv[u] = p + u < p1 ? val[p + u] : 0.0;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) r[u] = cc[u] != cc[u + 1] ? find(cc[u]) : -1;   // (see last_of_run)
+                for (int u = 0; u < 4; ++u) {
+                    r[u] = find(cc[u]);
+                    repeats |= r[u] >= 0 && r[u] == last;
+                    last = r[u];
+                }
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
                     if (r[u] >= 0) {
                         M[(size_t)c * ld + r[u]] = vv[u];
-                        x.flip(r[u]);
-                        mxb = max(mxb, absbits(vv[u]));
+                        x.set(r[u]);
+                        cmax = max(cmax, absbits(vv[u]));
                     }
             }
+            if (repeats) {   // the last value of a repeated column stands (see last_of_run)
+                cmax = 0;
+                for (int r = 0; r < np; ++r)
+                    if (x.has(r)) cmax = max(cmax, absbits(M[(size_t)c * ld + r]));
+            }
+            mxb = max(mxb, cmax);
             cm[t] = x;
         }
         if (has)
             for (int p = rowptr[i] + g; p < rowptr[i + 1]; p += G) {
-                const int r = last_of_run(p, rowptr[i + 1], col) ? find(col[p]) : -1;
-                if (r >= 0) ys[r] = -val[p];
+                const int r = find(col[p]);
+                if (r >= 0 && last_of_run(p, rowptr[i + 1], col)) ys[r] = -val[p];
             }
         __syncwarp();
         double y[R];
