@@ -1764,30 +1764,36 @@ __global__ void __launch_bounds__(PART_BS) k_class_scatter(int n, const int8_t *
     list[off[c * nblk + blockIdx.x] + before + rank_in_warp] = i;
 }
 
-__global__ void k_class_counts(int nclass, int nblk, const int *off, int *out) {
+__global__ void k_class_counts(int nclass, int nblk, const int *off, const int *extra, int nextra, int *out) {
     const int c = threadIdx.x;
     if (c <= nclass) out[c] = off[c * nblk];   // class starts, and the total
+    else if (c - nclass - 1 < nextra) out[c] = extra[c - nclass - 1];
 }
 
-void partition_by_class(const int8_t *cls, int n, int nclass, int *list, int *start, int *count, cudaStream_t s) {
-    PR_REQUIRE(nclass >= 1 && nclass <= PART_MAXC, PAIR_ERR_DEVICE, "partition_by_class: too many classes");
+// extra (device, nextra values): read together with the counts into hextra
+void partition_by_class(const int8_t *cls, int n, int nclass, int *list, int *start, int *count, cudaStream_t s,
+                        const int *extra = nullptr, int nextra = 0, int *hextra = nullptr) {
+    PR_REQUIRE(nclass >= 1 && nclass <= PART_MAXC && nclass + 1 + nextra <= 32, PAIR_ERR_DEVICE,
+               "partition_by_class: too many classes");
     if (n <= 0) {
         for (int c = 0; c < nclass; ++c) { start[c] = 0; count[c] = 0; }
+        for (int k = 0; k < nextra; ++k) hextra[k] = 0;
         return;
     }
     const int nblk = (int)blocks_for(n, PART_BS);
     const int nh = nclass * nblk;
-    int *hist = dmalloc<int>(nh, s), *off = dmalloc<int>(nh + 1, s), *cs = dmalloc<int>(nclass + 1, s);
+    int *hist = dmalloc<int>(nh, s), *off = dmalloc<int>(nh + 1, s), *cs = dmalloc<int>(nclass + 1 + nextra, s);
     k_class_hist<<<nblk, PART_BS, 0, s>>>(n, cls, nclass, nblk, hist);
     PR_LAUNCH();
     scan_exclusive(hist, off, nh, s, false);
     k_class_scatter<<<nblk, PART_BS, 0, s>>>(n, cls, nclass, nblk, off, list);
     PR_LAUNCH();
-    k_class_counts<<<1, 32, 0, s>>>(nclass, nblk, off, cs);
+    k_class_counts<<<1, 32, 0, s>>>(nclass, nblk, off, extra, nextra, cs);
     PR_LAUNCH();
-    int h[PART_MAXC + 1];
-    d2h(h, cs, nclass + 1, s);
+    int h[32];
+    d2h(h, cs, nclass + 1 + nextra, s);
     for (int c = 0; c < nclass; ++c) { start[c] = h[c]; count[c] = h[c + 1] - h[c]; }
+    for (int k = 0; k < nextra; ++k) hextra[k] = h[nclass + 1 + k];
     dfree(hist, s);
     dfree(off, s);
     dfree(cs, s);
@@ -2332,10 +2338,10 @@ void build_hierarchy(Hier &h) {
             PR_LAUNCH();
             int hc[LAIR_CLASSES], hstart[LAIR_CLASSES];
             int *list = dmalloc<int>(nc, s);
-            partition_by_class(ccls, nc, LAIR_CLASSES, list, hstart, hc, s);
+            int cls_n[LAIR_CLASSES] = {4, 6, 8, 12, 16, 24, 32, 48, 64};   // then the largest at hand
+            partition_by_class(ccls, nc, LAIR_CLASSES, list, hstart, hc, s, dbmax, LAIR_BIG - LAIR_SLOT,
+                               cls_n + LAIR_SLOT);
             dfree(ccls, s);
-            int cls_n[LAIR_CLASSES] = {4, 6, 8, 12, 16, 24, 32, 48, 64, 0, 0, 0};
-            if (hc[LAIR_SLOT] || hc[LAIR_SLOT + 1]) d2h(cls_n + LAIR_SLOT, dbmax, LAIR_BIG - LAIR_SLOT, s);
             dfree(dbmax, s);
             // blocks of one to four warps, so that the shared memory of an SM fills evenly
             auto mask_bin = [&](int c, auto kern, int G, int R) {
