@@ -64,10 +64,12 @@ typedef struct pair_hier_s *pair_hier;
  *  phi_A         filter applied to every coarse operator, diagonal kept (0 = off)
  *  max_levels    level cap (including the finest)
  *  max_coarse    a level with at most this many rows is the coarsest
- *  coarse_sweeps pointwise Jacobi sweeps from zero on the coarsest level (coarsest
- *                levels of at most 128 rows per matrix apply them as one dense product
- *                formed in the setup; up to 40 KB they run in one CTA per matrix in
- *                shared memory, larger ones grid-wide, one launch per sweep)
+ *  coarse_sweeps pointwise Jacobi sweeps from zero on the coarsest level.  Chosen for
+ *                all of a batch's matrices that end on the same level: if one of them
+ *                takes more than 40 KB there (entries, vectors, row pointer), the sweeps
+ *                run grid-wide, one launch each; else, if all have at most 128 rows and
+ *                their products fit 256 MB together, as one dense product formed in the
+ *                setup; else in one CTA per matrix in shared memory
  *  seed          PMIS key hash seed
  *  precision     0: hierarchy values and V-cycle in FP64;
  *                1: FP32 hierarchy and V-cycle under FP64 iterative refinement

@@ -361,9 +361,10 @@ void inner_enable(Hier &h);
 void residual_outer(Hier &h, const double *b, const double *x, double tol, bool zero_x = false);
 void inner_cycle(Hier &h, ProfSlot *ps);
 void fold_delta(Hier &h, double *x);
+// cB of a level whose segments are all small (setup; sweeps stay where it does not fit)
+void coarsest_dense(Hier &h, Level &L);
 // double-float mode (h.dd): b and x to pairs before a solve, x back after it; the
 // residual and the final relaxation then work on h.b_dd / h.x_dd
-void coarsest_dense(Hier &h, Level &L);   // cB of a level whose segments are all small
 void dd_enable(Hier &h);            // bsr_dd from bsr64 (frees bsr64), vectors
 void split0_enable(Hier &h);        // v0 from bsr32 (frees bsr32)
 void dd_load(Hier &h, const double *b, const double *x);

@@ -2,7 +2,8 @@
 // Jacobi).  Correction form with zero initial guess on every level:
 //   level 0: r = b - A x (FP64, cast to the cycle precision T), per-matrix ||r||
 //   down:    b_{l+1} = R_l b_l, R row = [Z_i, 1] (restriction of the residual)
-//   coarsest: coarse_sweeps Jacobi sweeps from 0 (one CTA per matrix segment)
+//   coarsest: coarse_sweeps Jacobi sweeps from 0 (small segments: as one dense product;
+//            up to CS_SMEM bytes: one CTA per matrix segment; larger: grid-wide)
 //   up:      y_l = P x_{l+1} (one-point: y_i = x_{l+1}[pmap(i)]); on the levels that relax
 //            from SELL copies y exists on the C rows only, and the first F sweep reads
 //            x_{l+1} through its entries' P columns
@@ -102,9 +103,11 @@ __device__ __forceinline__ HexFaces<T> hex_faces(int n, long long E, int m, int 
     return f;
 }
 
-// The same without loads ahead: each face's values and gathers together.  On launches of
-// many waves this keeps fewer values live at once than loading the three faces first
-// (64^3, 15 directions: FP32 residual 312 against 380 us, FP64 629 against 783 us).
+// The same without loads ahead: each face's values and gathers together.  On the large
+// launches of the two residuals this keeps fewer values live at once than loading the three
+// faces first (64^3, 15 directions: FP32 residual 312 against 380 us, FP64 629 against 783
+// us).  (k_relax0_split loads its three faces first in both forms: they lie side by side in
+// its copy, and the form did not slow it down, 32 sweeps of 32^3 S4 1.57 -> 1.45 ms.)
 template <class T, class TV>
 __device__ __forceinline__ T hex_offdiag(int n, long long E, int m, int e, int a, const int *idx, const int8_t *dsign,
                                          const T *vals, const TV *v) {
@@ -1156,6 +1159,9 @@ const double *lv_dinv<double>(const Level &L) { return L.dinv; }
 //   24^3 x 4, one solve      4.23     3.63     3.64     3.70
 //   24^3 S4 gradient       328.8    317.0    314.8    319.9
 //   32^3 S4                179.6    181.3    180.1    193.5
+// Single runs; two runs of one build differ by 0.5 to 3%.  One limit for every kernel and
+// both precisions: the tet case would like none and the single solve 6, by less than a run's
+// spread, and the large launches of 32^3 S4 need one.
 constexpr int AHEAD_BLOCKS_PER_SM = 12;
 bool load_ahead(long long blocks, int sms) { return blocks <= (long long)AHEAD_BLOCKS_PER_SM * sms; }
 
